@@ -381,7 +381,7 @@ __device__ void task_col2(const BatchDisc<R> &D, int cb, unsigned char *smem, un
 }
 
 // Column m = 0 (the packed m = 0 and m = nphi/2 real columns).  Every group
-// computes it; group 0 stores.  Same arithmetic as col0_path.
+// computes it; group 0 stores.  Same products as col0_output (sg_cols.cuh).
 template <typename R, int NS>
 __device__ void task_col0(const BatchDisc<R> &D, unsigned char *smem)
 {

@@ -21,109 +21,62 @@ __device__ __forceinline__ C spec_at(const C *col, int k, int H, bool upper)
 
 // Column m = 0 holds the packed (m = 0, m = nphi/2) pair of real columns:
 // Z = A + i B, so P = A S0 + i B SN = ((Z + Z*(-k)) S0 + (Z - Z*(-k)) SN) / 2.
-template <typename R, int NS>
-__device__ __noinline__ void col0_path(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab,
-                                       cplx<R> *__restrict__ oh, int nr, int N, uint32_t outmask,
-                                       const cplx<R> *__restrict__ tw, cplx<R> *xb, cplx<R> *spec)
+//
+// Every requested output of column 0 has a CTA of its own (the first CTAs of
+// the grid): NS forward transforms, the products and one inverse transform, so
+// no CTA's chain is longer than another column's.  One CTA for all outputs is
+// a chain of up to 3 NS (NS + 1) transforms with its table loads between them,
+// which set the time of every small column pass: 256 x 512 gas + dust 50 us,
+// 1024 x 2048 accelerations 48 us (LC: compile-time length, as in k_cols).
+// The two table columns of each source go to L2 while the forward transform
+// runs; Z*(L - k) comes through the exchange buffer.
+template <typename R, int NS, int LC>
+__device__ __noinline__ void col0_output(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab,
+                                         cplx<R> *__restrict__ oh, int nr, int N, int q,
+                                         const cplx<R> *__restrict__ tw, cplx<R> *xb)
 {
     using C = cplx<R>;
-    const int L = 2 * nr, T = L >> 4, H = nr, P = tab_pitch(nr);
-    const int t = threadIdx.x;
-    C v[16];
+    const int L = LC > 0 ? LC : 2 * nr, T = L >> 4, H = L >> 1, P = tab_pitch(H);
+    const int t = threadIdx.x, b = q / 3, c = q - 3 * b;
+    if (t < 2 * NS)
+        prefetch_l2_bulk(tab + (((size_t)((t >> 1) * NS + b) * 3 + c) * (N + 1) + (size_t)(t & 1) * N) * P,
+                         (unsigned)(P * sizeof(C)));
+    griddep_wait();                                // the row spectra are complete from here on
+    C acc[16];
+#pragma unroll 1
     for (int a = 0; a < NS; ++a) {
+        C v[16];
         const C *col = sh + (size_t)a * N * nr;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = ld_cg_hint(col + blk(0, t + T * e, nr), l2_evict_first());
+        for (int e = 0; e < 8; ++e) v[e] = ld_cg_hint(col + blk(0, t + T * e, nr), l2_evict_last());
 #pragma unroll
         for (int e = 8; e < 16; ++e) v[e] = mkc<C>(0, 0);
-        fft_reg<true>(v, L, T, t, xb, tw);
+        fft_any<true, LC, true>(v, L, T, t, xb, tw);
+        __syncthreads();                           // the transform's last exchange reads are done
 #pragma unroll
-        for (int e = 0; e < 16; ++e) spec[a * L + t + T * e] = v[e];
-    }
-    __syncthreads();
-    for (int b = 0; b < NS; ++b) {
-        for (int c = 0; c < 3; ++c) {
-            if (!((outmask >> (3 * b + c)) & 1u)) continue;
+        for (int e = 0; e < 16; ++e) xb[pidx(t + T * e)] = v[e];
+        __syncthreads();
+        const C *t0 = tab + ((size_t)((a * NS + b) * 3 + c) * (N + 1)) * P;
+        const C *tn = t0 + (size_t)N * P;
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int k = t + T * e;
-                C acc = mkc<C>(0, 0);
-                for (int a = 0; a < NS; ++a) {
-                    const C *t0 = tab + ((size_t)((a * NS + b) * 3 + c) * (N + 1)) * P;
-                    const C *tn = t0 + (size_t)N * P;
-                    const C Z = spec[a * L + k];
-                    const C Zm = cconj(spec[a * L + ((L - k) & (L - 1))]);
-                    C S0 = spec_at(t0, k, H, e >= 8), SN = spec_at(tn, k, H, e >= 8);
-                    if (c == 2) {
-                        S0 = cmul_mi(S0);
-                        SN = cmul_mi(SN);
-                    }
-                    acc = cadd(acc, cscale(cadd(cmul(cadd(Z, Zm), S0), cmul(csub(Z, Zm), SN)), (R)0.5));
-                }
-                v[e] = acc;
+        for (int e = 0; e < 16; ++e) {
+            const int k = t + T * e;
+            const C Z = v[e];
+            const C Zm = cconj(xb[pidx((L - k) & (L - 1))]);
+            C S0 = spec_at(t0, k, H, e >= 8), SN = spec_at(tn, k, H, e >= 8);
+            if (c == 2) {
+                S0 = cmul_mi(S0);
+                SN = cmul_mi(SN);
             }
-            fft_reg<false>(v, L, T, t, xb, tw);
-            C *o = oh + (size_t)(b * 3 + c) * N * nr;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) o[blk(0, t + T * e, nr)] = v[e];
+            const C p = cscale(cadd(cmul(cadd(Z, Zm), S0), cmul(csub(Z, Zm), SN)), (R)0.5);
+            acc[e] = a == 0 ? p : cadd(acc[e], p);
         }
+        __syncthreads();                           // before the next transform rewrites the buffer
     }
-}
-
-// LC > 0: compile-time column length (2 nr).
-// Column 0 of a plan that stages kernel spectra per step (no shared-memory
-// source spectra): each requested (target, component) step transforms the
-// packed source columns again and pairs Z(k) with Z*(L - k) through the
-// exchange buffer.  The same terms in the same order as col0_path, so the
-// same result; for gas + dust 18 transforms instead of 8, in one CTA of the
-// first wave.
-template <typename R, int NS>
-__device__ __noinline__ void col0_recompute(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab,
-                                            cplx<R> *__restrict__ oh, int nr, int N, uint32_t outmask,
-                                            const cplx<R> *__restrict__ tw, cplx<R> *xb)
-{
-    using C = cplx<R>;
-    const int L = 2 * nr, T = L >> 4, H = nr, P = tab_pitch(nr);
-    const int t = threadIdx.x;
-    for (int q = 0; q < 3 * NS; ++q) {
-        if (!((outmask >> q) & 1u)) continue;
-        const int b = q / 3, c = q % 3;
-        C acc[16];
+    fft_any<false, LC>(acc, L, T, t, xb, tw);
+    C *o = oh + (size_t)q * N * nr;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e] = mkc<C>(0, 0);
-        for (int a = 0; a < NS; ++a) {
-            C v[16];
-            const C *col = sh + (size_t)a * N * nr;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = ld_cg_hint(col + blk(0, t + T * e, nr), l2_evict_first());
-#pragma unroll
-            for (int e = 8; e < 16; ++e) v[e] = mkc<C>(0, 0);
-            fft_reg<true>(v, L, T, t, xb, tw);
-            __syncthreads();                   // the transform's last exchange reads are done
-#pragma unroll
-            for (int e = 0; e < 16; ++e) xb[pidx(t + T * e)] = v[e];
-            __syncthreads();
-            const C *t0 = tab + ((size_t)((a * NS + b) * 3 + c) * (N + 1)) * P;
-            const C *tn = t0 + (size_t)N * P;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int k = t + T * e;
-                const C Z = v[e];
-                const C Zm = cconj(xb[pidx((L - k) & (L - 1))]);
-                C S0 = spec_at(t0, k, H, e >= 8), SN = spec_at(tn, k, H, e >= 8);
-                if (c == 2) {
-                    S0 = cmul_mi(S0);
-                    SN = cmul_mi(SN);
-                }
-                acc[e] = cadd(acc[e], cscale(cadd(cmul(cadd(Z, Zm), S0), cmul(csub(Z, Zm), SN)), (R)0.5));
-            }
-            __syncthreads();                   // before the next transform rewrites the buffer
-        }
-        fft_reg<false>(acc, L, T, t, xb, tw);
-        C *o = oh + (size_t)(b * 3 + c) * N * nr;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) o[blk(0, t + T * e, nr)] = acc[e];
-    }
+    for (int e = 0; e < 8; ++e) o[blk(0, t + T * e, nr)] = acc[e];
 }
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
@@ -236,8 +189,9 @@ __device__ __forceinline__ void cols_pair_steps(const cplx<R> *__restrict__ sh, 
     }
 }
 
-// Column pass, one CTA per column m (LC: compile-time column length, 0 for
-// any; ST: staging as above).
+// Column pass: one CTA per requested output of column 0, then one CTA per
+// column m >= 1 (LC: compile-time column length, 0 for any; ST: staging as
+// above; outmask holds the requested outputs of this plan's fluids only).
 template <typename R, int NS, int LC, bool ST>
 __global__ void __launch_bounds__(cols_max_threads(NS, sizeof(R) == 8, LC, ST),
                                   cols_min_blocks(NS, sizeof(R) == 8, LC, ST))
@@ -251,16 +205,13 @@ k_cols(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<R> 
     const int L = 2 * nr, T = L >> 4, H = nr, P = tab_pitch(nr);
     C *xb = reinterpret_cast<C *>(smem_raw + 16);
     C *tb = reinterpret_cast<C *>(smem_raw + 16 + align16((size_t)padded_len(L) * sizeof(C)));
-    const int t = threadIdx.x, m = blockIdx.x;
+    const int t = threadIdx.x, nq = __popc(outmask), m = (int)blockIdx.x - nq + 1;
     griddep_launch();                     // the inverse rows may set up once every column CTA runs
     static_assert(!ST || sizeof(R) == 4, "per-step staging is FP32 only");
     constexpr bool PAIR = ST;
-    if (m == 0) {
-        // column 0 keeps its source spectra in the table area (recomputed
-        // per step when staging per step)
-        griddep_wait();
-        if constexpr (PAIR) col0_recompute<R, NS>(sh, tab, oh, nr, N, outmask, tw, xb);
-        else col0_path<R, NS>(sh, tab, oh, nr, N, outmask, tw, xb, tb);
+    if (m < 1) {
+        // column 0: CTA i computes the i-th requested output
+        col0_output<R, NS, LC>(sh, tab, oh, nr, N, (int)__fns(outmask, 0, (int)blockIdx.x + 1), tw, xb);
         return;
     }
     if constexpr (PAIR) {

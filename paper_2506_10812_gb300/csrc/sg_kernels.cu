@@ -69,13 +69,11 @@ size_t col_smem_bytes(int nr, int nsrc, bool f64, int staging)
     const int L = 2 * nr;
     const size_t xb = align16((size_t)padded_len(L) * esz);
     // per step: one (target, component) step of kernel spectra staged at a
-    // time, source spectra in registers, column 0 recomputed per step
+    // time, source spectra in registers
     if (cols_staging_steps(nr, nsrc, f64, staging)) return 16 + xb + (size_t)nsrc * tab_pitch(nr) * esz;
     const size_t tb = (size_t)nsrc * 3 * tab_pitch(nr) * esz;
     const size_t spec = nsrc == 2 ? (size_t)2 * L * esz : 0;   // gas + dust spectra live in shared memory
-    // column 0 keeps its source spectra in the table area instead
-    const size_t col0 = (size_t)nsrc * L * esz;
-    return 16 + xb + (tb > col0 ? tb : col0) + spec;
+    return 16 + xb + tb + spec;
 }
 
 size_t tabcol_smem_bytes(int L, bool) { return (size_t)padded_len(L) * 16; }
@@ -177,9 +175,9 @@ cudaError_t launch_cols(const void *sh, const void *tab, void *oh, int nr, int n
     const int N = nphi / 2, T = (2 * nr) / 16;
     const bool steps = cols_staging_steps(nr, nsrc, f64, staging);
     const size_t smem = col_smem_bytes(nr, nsrc, f64, steps ? 1 : 0);
-    const int grid = ncols > 0 && ncols < N ? ncols : N;
-    // whole 128-byte lines per source column (column 0 is read more than once
-    // by its CTA and never discarded)
+    const int grid = (ncols > 0 && ncols < N ? ncols : N) - 1 + __builtin_popcount(outmask);
+    // whole 128-byte lines per source column (column 0 is read by every
+    // output's CTA and never discarded)
     const bool dc = discard && BW == 1 && ((size_t)nr * 2 * sizeof(R)) % 128 == 0 && ((uintptr_t)sh & 127u) == 0;
     ColsKernel<R> kern;
     if constexpr (sizeof(R) == 4) kern = steps ? cols_kernel_steps(nsrc, 2 * nr) : cols_kernel_all<R>(nsrc, 2 * nr);
