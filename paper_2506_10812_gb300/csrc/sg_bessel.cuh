@@ -16,9 +16,17 @@
 //               exactly, so no digits are lost).
 // Measured against 30-digit references: FP64 <= 1e-15, FP32 <= 2.3e-7
 // relative over their ranges.
+//
+// Where a function is evaluated per pair of cells the representations above
+// are too long: FP64 units run at 1/64 of the FP32 rate here, and a quadrature
+// is 24 reciprocal square roots.  bessel_table and the tail polynomials
+// (sg_bessel_tab.cuh) take one short polynomial per function instead: FP64
+// 12 or 10 multiply-adds, FP32 5 or 4.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include "sg_bessel_tab.cuh"
 
 namespace sg {
 
@@ -48,33 +56,39 @@ __device__ __forceinline__ void bessel_weights_init(BesselWeights &bw)
     }
 }
 
+// the ascending series, x < 2
+__device__ __forceinline__ void k0e_D_series(double x, double &k0e, double &D)
+{
+    // K0 = -(ln(x/2) + gamma) I0 + sum_{k>=1} H_k y^k / (k!)^2,
+    // K1 = 1/x + ln(x/2) I1 - (x/4) sum_k (psi(k+1) + psi(k+2)) y^k / (k! (k+1)!),
+    // y = x^2/4, psi(k+1) = H_k - gamma.
+    const double gam = 0.57721566490153286061;
+    const double y = 0.25 * x * x;
+    const double L = log(0.5 * x);
+    double t0 = 1.0, t1 = 1.0, H = 0.0;
+    double I0 = 1.0, I1s = 1.0, S0 = 0.0;
+    double S1 = 1.0 - 2.0 * gam;   // k = 0 term: psi(1) + psi(2) = 1 - 2 gamma
+    for (int k = 1; k < 40; ++k) {
+        t0 *= y / ((double)k * k);
+        t1 *= y / ((double)k * (k + 1));
+        H += 1.0 / k;
+        I0 += t0;
+        I1s += t1;
+        S0 += H * t0;
+        S1 += (2.0 * H + 1.0 / (k + 1) - 2.0 * gam) * t1;
+        if (t0 < 1e-18 * I0) break;
+    }
+    const double K0 = -(L + gam) * I0 + S0;
+    const double K1 = 1.0 / x + L * (0.5 * x) * I1s - 0.25 * x * S1;
+    const double ex = exp(x);
+    k0e = ex * K0;
+    D = ex * (K1 - K0);
+}
+
 __device__ __forceinline__ void k0e_D_f64(double x, const BesselWeights &bw, double &k0e, double &D)
 {
     if (x < 2.0) {
-        // K0 = -(ln(x/2) + gamma) I0 + sum_{k>=1} H_k y^k / (k!)^2,
-        // K1 = 1/x + ln(x/2) I1 - (x/4) sum_k (psi(k+1) + psi(k+2)) y^k / (k! (k+1)!),
-        // y = x^2/4, psi(k+1) = H_k - gamma.
-        const double gam = 0.57721566490153286061;
-        const double y = 0.25 * x * x;
-        const double L = log(0.5 * x);
-        double t0 = 1.0, t1 = 1.0, H = 0.0;
-        double I0 = 1.0, I1s = 1.0, S0 = 0.0;
-        double S1 = 1.0 - 2.0 * gam;   // k = 0 term: psi(1) + psi(2) = 1 - 2 gamma
-        for (int k = 1; k < 40; ++k) {
-            t0 *= y / ((double)k * k);
-            t1 *= y / ((double)k * (k + 1));
-            H += 1.0 / k;
-            I0 += t0;
-            I1s += t1;
-            S0 += H * t0;
-            S1 += (2.0 * H + 1.0 / (k + 1) - 2.0 * gam) * t1;
-            if (t0 < 1e-18 * I0) break;
-        }
-        const double K0 = -(L + gam) * I0 + S0;
-        const double K1 = 1.0 / x + L * (0.5 * x) * I1s - 0.25 * x * S1;
-        const double ex = exp(x);
-        k0e = ex * K0;
-        D = ex * (K1 - K0);
+        k0e_D_series(x, k0e, D);
     } else if (x < 40.0) {
         const double q = 0.25 / x;
         double s0 = 0.5, s1 = 0.0;
@@ -136,6 +150,58 @@ __device__ __forceinline__ void k0e_D_f32(float x, const BesselWeights &bw, floa
         }
         k0e = s * s0;
         D = s * sd;
+    }
+}
+
+// K0e(x) and E(x) = x D(x) from the quarter-octave tables, 2^-20 <= x < 16
+// (bessel_in_table).  The index and the argument come from the bits of x; a
+// warp's lanes mostly share an entry, so the loads are broadcasts from L1.
+__device__ __forceinline__ bool bessel_in_table(float x) { return x >= 0x1p-20f && x < 16.0f; }
+__device__ __forceinline__ bool bessel_in_table(double x) { return x >= 0x1p-20 && x < 16.0; }
+__device__ __forceinline__ void bessel_table(float x, float &k0e, float &E)
+{
+    const int b = __float_as_int(x);
+    const float4 *c = reinterpret_cast<const float4 *>(&BT_32[(b >> 21) - 4 * (127 + BT_LO)][0][0]);
+    const float t = __int_as_float((b & 0x007FFFFF) | 0x3F800000) - __int_as_float((b & 0x00600000) | 0x3F900000);
+    const float4 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
+    k0e = fmaf(fmaf(fmaf(fmaf(fmaf(c1.y, t, c1.x), t, c0.w), t, c0.z), t, c0.y), t, c0.x);
+    E = fmaf(fmaf(fmaf(fmaf(fmaf(c2.w, t, c2.z), t, c2.y), t, c2.x), t, c1.w), t, c1.z);
+}
+__device__ __forceinline__ void bessel_table(double x, double &k0e, double &E)
+{
+    const int hi = __double2hiint(x);
+    const double *c = &BT_64[(hi >> 18) - 4 * (1023 + BT_LO)][0][0];
+    const double t = __hiloint2double((hi & 0x000FFFFF) | 0x3FF00000, __double2loint(x)) -
+                     __hiloint2double((hi & 0x000C0000) | 0x3FF20000, 0);
+    double a = __ldg(c + 12), b = __ldg(c + 25);
+#pragma unroll
+    for (int k = 11; k >= 0; --k) {
+        a = fma(a, t, __ldg(c + k));
+        b = fma(b, t, __ldg(c + 13 + k));
+    }
+    k0e = a;
+    E = b;
+}
+// The tails in z = 1/x <= 1/16: K0e = sqrt(pi z / 2) S0, E = sqrt(pi z / 2) Q / 2.
+constexpr double BESSEL_ZTAIL = 0.0625;
+__device__ __forceinline__ void bessel_tail(float z, float &S0, float &Q)
+{
+    S0 = BT_S0_32[4];
+    Q = BT_Q_32[4];
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+        S0 = fmaf(S0, z, BT_S0_32[k]);
+        Q = fmaf(Q, z, BT_Q_32[k]);
+    }
+}
+__device__ __forceinline__ void bessel_tail(double z, double &S0, double &Q)
+{
+    S0 = BT_S0_64[9];
+    Q = fma(BT_Q_64[10], z, BT_Q_64[9]);
+#pragma unroll
+    for (int k = 8; k >= 0; --k) {
+        S0 = fma(S0, z, BT_S0_64[k]);
+        Q = fma(Q, z, BT_Q_64[k]);
     }
 }
 

@@ -12,6 +12,32 @@
 //     e_phi . (r - r') = r' sin psi,
 // using per-lag tables built in FP64, so FP32 keeps full relative precision
 // for the nearest neighbours (no cancellation in r - r').
+//
+// Bound and decomposition.  The sum is bound by the FP pipes (FP64: 1/64 of the
+// FP32 lane rate), so the kernel is built to leave few operations per pair.  A
+// pair's geometry depends on the row pair and on dj alone, its scale height on
+// the two cells.  With lengths in units of sqrt(r r') (sigma = s^2 / (r r'),
+// eta = H^2 / (r r')) and z = 1/X = 4 (eta_a + eta_b) / sigma,
+//     Phi term = m / s S0(z),   force term = m / s^3 (r - r') Q(z),
+// S0 and Q the tails of the Bessel functions (1 at z = 0: the Newtonian
+// limit).  So a CTA owns KT x blockDim targets of one row and walks the source
+// rows; per source row it tabulates, for a tile of lags dj, (4 / sigma,
+// sigma^-1/2 and the two sigma^-3/2 weights) once for all its targets, stages
+// the window of sources the tile meets, and then runs over dj: the lag's
+// entry is one broadcast, a target's source is at a fixed distance (conflict-
+// free), and a pair with z <= 1/16 costs 15 operations (FP32; 27 in FP64)
+// instead of a Bessel evaluation by branch (about 360).  Lags that may hold a larger z (a bound from the
+// tile's largest scale heights; they lie around dj = 0) take the table
+// polynomials instead; every lane of a warp is on the same lag, so the two paths do not diverge.
+// Sums: 16 lags in a register, then Kahan-compensated.  Measured (solve): 128 x 256 gas + dust FP32
+// 112.6 -> 4.34 ms (0.99 Tpair/s; 15 operations at the FMA pipes' 37 Tlane/s would be 2.3), 61 x 150
+// gas FP64 227 -> 6.89 ms (12.2 Gpair/s of the 21 that 27 operations allow), against one thread per
+// target with the Bessel functions by branch; errors against 64 bits as before (1.8e-7, 3.5e-15).
+//
+// The source rows are split over the CTAs of a cluster, whose partial sums
+// are added through distributed shared memory in rank order (no workspace, the
+// same bits every time).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -24,6 +50,8 @@
 #include "sg_internal.h"
 
 namespace sg {
+
+namespace cg = cooperative_groups;
 
 template <typename R> struct pair_of;
 template <> struct pair_of<float> { using type = float2; };
@@ -40,47 +68,253 @@ template <typename R> struct Acc {
     }
 };
 
-template <typename R>
-__device__ __forceinline__ void k0e_D_any(R x, const BesselWeights &bw, R &k0e, R &D);
-template <>
-__device__ __forceinline__ void k0e_D_any<double>(double x, const BesselWeights &bw, double &k0e, double &D)
+constexpr int DLT = 128;          // lags per tile
+constexpr int DGROUP = 16;        // lags per uncompensated partial sum
+constexpr int DMAXT = 256;        // threads per CTA, at most
+
+template <typename R> struct __align__(16) LagFar { R iz, w1, wr, wp; };   // 4 / sigma, and the weights
+template <typename R> struct __align__(2 * sizeof(R)) Duo { R x, y; };
+
+// shared memory of a CTA of T threads and KT targets each; the partial sums
+// overlay the tables at the end
+template <typename R> constexpr size_t direct_smem(int T, int KT)
 {
-    k0e_D_f64(x, bw, k0e, D);
+    const size_t tab = DLT * (sizeof(LagFar<R>) + sizeof(Duo<R>)) + (size_t)(T * KT + DLT) * sizeof(Duo<R>);
+    const size_t red = (size_t)3 * T * KT * sizeof(R);
+    return tab > red ? tab : red;
 }
-template <>
-__device__ __forceinline__ void k0e_D_any<float>(float x, const BesselWeights &bw, float &k0e, float &D)
+
+// 1 / sqrt(x) to rounding (the FP32 instruction alone is off by 2 ulp, and the
+// force takes its cube)
+__device__ __forceinline__ float rsqrt_r(float x)
 {
-    if (x < 1.0f) {   // log singularity region: FP64
+    const float y = rsqrtf(x), e = fmaf(-x * y, y, 1.0f);
+    return fmaf(0.5f * y, e, y);
+}
+__device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
+
+// One pair by its own scale height: (K0e, E) at z = 1 / X, any z.
+template <typename R>
+__device__ __forceinline__ void pair_bessel(R z, R &k0e, R &E)
+{
+    if (z <= (R)BESSEL_ZTAIL) {
+        R S0, Q;
+        bessel_tail(z, S0, Q);
+        const R s = sqrt((R)1.5707963267948966192 * z);
+        k0e = s * S0;
+        E = (R)0.5 * s * Q;
+        return;
+    }
+    const R X = (R)1 / z;
+    if (bessel_in_table(X)) {
+        bessel_table(X, k0e, E);
+    } else {                                   // X < 2^-20, or not a number
         double a, b;
-        k0e_D_f64((double)x, bw, a, b);
-        k0e = (float)a;
-        D = (float)b;
-    } else {
-        k0e_D_f32(x, bw, k0e, D);
+        k0e_D_series((double)X, a, b);
+        k0e = (R)a;
+        E = (R)(b * (double)X);
     }
 }
 
-constexpr int DT = 256;   // targets per CTA and sources per shared-memory tile
-// FP32: compiled for 4 resident CTAs per SM (64 registers, a few spilled):
-// 256 x 512 gas + dust solve 708 -> 641 ms against the unbounded 94-register
-// build at 2 CTAs per SM (2 and 3 CTAs per SM: 754 and 751 ms); bit-identical.
-#ifndef SG_DIRECT_MINB
-#define SG_DIRECT_MINB 4
-#endif
-
-template <typename R>
-__global__ void __launch_bounds__(DT, sizeof(R) == 4 ? SG_DIRECT_MINB : 1)
-k_direct(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__restrict__ sig_d,
+template <typename R, int KT>
+__global__ void __launch_bounds__(DMAXT)
+k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R *__restrict__ sig_d,
          const R *__restrict__ Hg, const R *__restrict__ Hd, R h_g, R h_d, int tgt, R *phi, R *gr,
          R *gphi, const typename pair_of<R>::type *__restrict__ geo_i,
          const typename pair_of<R>::type *__restrict__ geo_j, const R *__restrict__ rcen, R dudphi,
          unsigned int *flag)
 {
     using P2 = typename pair_of<R>::type;
-    __shared__ BesselWeights bw;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    LagFar<R> *lagF = reinterpret_cast<LagFar<R> *>(smem_raw);
+    Duo<R> *lagN = reinterpret_cast<Duo<R> *>(lagF + DLT);       // (e_r, e_phi) geometry over r'
+    Duo<R> *win = lagN + DLT;                                    // (mass / sqrt(r r'), eta_a)
+    __shared__ unsigned s_bmax, s_amax[2];                       // largest |H_b| / r and eta_a, as their bits
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int t = threadIdx.x, T = blockDim.x, TJ = KT * T, lane = t & 31;
+    const int unit = blockIdx.x / S, i = unit / nchunk, j0 = (unit - i * nchunk) * TJ;
+    const R r = rcen[i];
+    const R *Hb_f = tgt == 0 ? Hg : Hd;
+    const R hb = tgt == 0 ? h_g : h_d;
+    R Hb[KT];
+    if (t == 0) {
+        s_bmax = 0u;
+        s_amax[0] = 0u;
+    }
+    __syncthreads();
+    {
+        float mx = 0.f;
+        bool nan = false;
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+            const int j = min(j0 + t + k * T, nphi - 1);        // past the row: a copy of its last target
+            Hb[k] = Hb_f ? Hb_f[(size_t)i * nphi + j] : hb * r;
+            const float h = fabsf((float)(Hb[k] / r));
+            nan |= h != h;
+            mx = fmaxf(mx, h);
+        }
+        const unsigned m = __reduce_max_sync(0xffffffffu, nan ? 0x7fc00000u : __float_as_uint(mx));
+        if (lane == 0) atomicMax(&s_bmax, m);
+    }
+    Acc<R> agr[KT], agp[KT], aph[KT];
+    int tile = 0;
+    const int nsrc_fluids = sig_d ? 2 : 1;
+    for (int a = 0; a < nsrc_fluids; ++a) {
+        const R *sig = a == 0 ? sig_g : sig_d;
+        const R *Ha_f = a == 0 ? Hg : Hd;
+        const R ha = a == 0 ? h_g : h_d;
+        for (int i2 = rank; i2 < nr; i2 += S) {
+            const R rr = rcen[i2];
+            const P2 gi = geo_i[i - i2 + nr - 1];                // (sinh^2(D/2), expm1(D))
+            const R q = (R)1 / sqrt(r * rr);
+            R eb[KT];
+#pragma unroll
+            for (int k = 0; k < KT; ++k) {
+                const R h = Hb[k] * q;
+                eb[k] = h * h;
+            }
+            for (int d0 = 0; d0 < nphi; d0 += DLT, ++tile) {
+                const int nlag = min(DLT, nphi - d0);
+                __syncthreads();                                 // the previous tile is done with
+                if (t == 0) s_amax[(tile + 1) & 1] = 0u;
+                // target slot x and lag d of the tile meet the source at window slot x - d + DLT - 1
+                float mx = 0.f;
+                bool nan = false;
+                for (int w = DLT - nlag + t; w < TJ + DLT - 1; w += T) {
+                    int jj = (j0 - d0 + w - (DLT - 1)) % nphi;
+                    if (jj < 0) jj += nphi;
+                    const size_t src = (size_t)i2 * nphi + jj;
+                    const R h = (Ha_f ? Ha_f[src] : ha * rr) * q, e = h * h;
+                    win[w] = {(G * sig[src] * rr * rr * dudphi) * q, e};
+                    const float ef = (float)e;
+                    nan |= ef != ef;
+                    mx = fmaxf(mx, ef);
+                }
+                const unsigned m = __reduce_max_sync(0xffffffffu, nan ? 0x7fc00000u : __float_as_uint(mx));
+                if (lane == 0) atomicMax(&s_amax[tile & 1], m);
+                for (int l = t; l < nlag; l += T) {
+                    const P2 gj = geo_j[d0 + l];                 // (sin^2(psi/2), sin psi)
+                    const R sg = (R)4 * (gi.x + gj.x);
+                    const R er = gi.y + (R)2 * gj.x;
+                    const R i1 = (R)1 / sqrt(sg), i3 = i1 / sg;
+                    lagF[l] = {(R)4 / sg, i1, i3 * er, i3 * gj.y};
+                    lagN[l] = {er, gj.y};
+                }
+                __syncthreads();
+                // [lo, hi): the lags whose pairs all have z <= 1/16 and whose
+                // weights are ordinary numbers; 4 / sigma falls towards dj = nphi / 2
+                int lo = 0, hi = nlag;
+                {
+                    const float hq = __uint_as_float(s_bmax) * (float)(r * q);
+                    const float lim = 1.001f * (__uint_as_float(s_amax[tile & 1]) + hq * hq);
+                    for (int l0 = 0; l0 < nlag; l0 += 32) {
+                        const int l = l0 + lane;
+                        bool near = false;
+                        if (l < nlag) {
+                            const float iz = (float)lagF[l].iz;
+                            near = !(iz * lim <= (float)BESSEL_ZTAIL && iz < 1e20f && iz > 1e-20f);
+                        }
+                        const bool first = 2 * (d0 + l) <= nphi;
+                        const unsigned nf = __ballot_sync(0xffffffffu, near && first);
+                        const unsigned ns = __ballot_sync(0xffffffffu, near && !first);
+                        if (nf) lo = l0 + 32 - __clz(nf);
+                        if (ns) hi = min(hi, l0 + __ffs(ns) - 1);
+                    }
+                }
+                const Duo<R> *wt = win + t + DLT - 1;
+                for (int g0 = lo; g0 < hi; g0 += DGROUP) {
+                    R sp[KT] = {}, sr[KT] = {}, sa[KT] = {};
+                    const int g1 = min(g0 + DGROUP, hi);
+#pragma unroll 4
+                    for (int d = g0; d < g1; ++d) {
+                        const LagFar<R> L = lagF[d];
+#pragma unroll
+                        for (int k = 0; k < KT; ++k) {
+                            const Duo<R> s = wt[k * T - d];
+                            R S0, Q;
+                            bessel_tail((s.y + eb[k]) * L.iz, S0, Q);
+                            sp[k] = fma(s.x, S0 * L.w1, sp[k]);
+                            Q *= s.x;
+                            sr[k] = fma(Q, L.wr, sr[k]);
+                            sa[k] = fma(Q, L.wp, sa[k]);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < KT; ++k) {
+                        aph[k].add(sp[k]);
+                        agr[k].add(sr[k]);
+                        agp[k].add(sa[k]);
+                    }
+                }
+                const R c_force = (R)(0.125 * 0.56418958354775628695);   // 1 / (8 sqrt(pi))
+                const R c_pot = (R)(0.5 * 0.56418958354775628695);       // 1 / (2 sqrt(pi))
+#pragma unroll 1
+                for (int d = 0; d < nlag; ++d) {
+                    if (d == lo && lo < hi) d = hi;
+                    if (d >= nlag) break;
+                    if (i2 == i && d0 + d == 0) continue;        // self cell excluded
+                    const R iz = lagF[d].iz;
+                    const Duo<R> g = lagN[d];
+#pragma unroll
+                    for (int k = 0; k < KT; ++k) {
+                        const Duo<R> s = wt[k * T - d];
+                        const R eta = s.y + eb[k], z = eta * iz;
+                        R k0e, E;
+                        pair_bessel(z, k0e, E);
+                        const R invH = rsqrt_r((R)0.5 * eta);
+                        const R f = s.x * (E * z) * c_force * invH * invH * invH;   // G m K / s
+                        agr[k].add(f * g.x);
+                        agp[k].add(f * g.y);
+                        aph[k].add(s.x * k0e * c_pot * invH);
+                    }
+                }
+            }
+        }
+    }
+    // partial sums of the cluster's ranks, in rank order
+    R *red = reinterpret_cast<R *>(smem_raw);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < KT; ++k) {
+        red[t + k * T] = aph[k].s;
+        red[TJ + t + k * T] = agr[k].s;
+        red[2 * TJ + t + k * T] = agp[k].s;
+    }
+    cluster.sync();
+    const R inv_r = (R)1 / r;
+    bool bad = false;
+    for (int x = rank * T + t; x < 3 * TJ; x += S * T) {
+        const int c = x / TJ, j = j0 + x - c * TJ;
+        if (j >= nphi) continue;
+        Acc<R> v;
+        for (int p = 0; p < S; ++p) v.add(*cluster.map_shared_rank(red + x, p));
+        const R o = c == 0 ? -v.s : -v.s * inv_r;
+        R *out = c == 0 ? phi : c == 1 ? gr : gphi;
+        if (out) out[(size_t)i * nphi + j] = o;
+        bad |= !isfinite(o);
+    }
+    if (flag && bad) atomicOr(flag, 1u);
+    cluster.sync();                                              // no CTA leaves while another reads its sums
+}
+
+// Short rows (nphi < kDirectRowMin): one thread per target over all sources,
+// the pair terms in the same variables.  A row kernel's warp would own one row
+// pair's few pairs and spend its time on the tables.  The line: at nphi = 8 the
+// rows take 0.042 against 0.164 ms (50 rows) and 5.98 against 5.45 (2000 rows),
+// at nphi = 4 0.054 against 0.165 (100 rows) but 12.8 against 4.1 (3000 rows).
+constexpr int DT = 256;   // targets per CTA and sources per shared-memory tile
+template <typename R>
+__global__ void __launch_bounds__(DT)
+k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__restrict__ sig_d,
+               const R *__restrict__ Hg, const R *__restrict__ Hd, R h_g, R h_d, int tgt, R *phi, R *gr,
+               R *gphi, const typename pair_of<R>::type *__restrict__ geo_i,
+               const typename pair_of<R>::type *__restrict__ geo_j, const R *__restrict__ rcen, R dudphi,
+               unsigned int *flag)
+{
+    using P2 = typename pair_of<R>::type;
     __shared__ R s_r[DT], s_m[DT], s_H2[DT];
     __shared__ int s_i[DT], s_j[DT];
-    bessel_weights_init(bw);
     const int ncell = nr * nphi;
     const int tid = blockIdx.x * DT + threadIdx.x;
     const bool valid = tid < ncell;
@@ -125,22 +359,53 @@ k_direct(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__restrict
                 const R rr = s_r[q];
                 const R s2 = (R)4 * r * rr * (gi.x + gj.x);
                 const R H2 = (R)0.5 * (s_H2[q] + Hb2);
-                const R X = s2 / ((R)8 * H2);
-                R k0e, D;
-                k0e_D_any<R>(X, bw, k0e, D);
-                const R invH = (R)1 / sqrt(H2);
-                const R f = -s_m[q] * D * c_force * invH * invH * invH;   // -G m K / s
+                const R z = (R)8 * H2 / s2;
+                R k0e, E;
+                pair_bessel(z, k0e, E);
+                const R invH = rsqrt_r(H2);
+                const R f = s_m[q] * (E * z) * c_force * invH * invH * invH;   // G m K / s
                 agr.add(f * rr * (gi.y + (R)2 * gj.x));
                 agp.add(f * rr * gj.y);
-                aph.add(-s_m[q] * k0e * c_pot * invH);
+                aph.add(s_m[q] * k0e * c_pot * invH);
             }
         }
     }
     if (!valid) return;
-    if (phi) phi[tid] = aph.s;
-    if (gr) gr[tid] = agr.s;
-    if (gphi) gphi[tid] = agp.s;
+    if (phi) phi[tid] = -aph.s;
+    if (gr) gr[tid] = -agr.s;
+    if (gphi) gphi[tid] = -agp.s;
     if (flag && !(isfinite(aph.s) && isfinite(agr.s) && isfinite(agp.s))) atomicOr(flag, 1u);
+}
+constexpr int kDirectRowMin = 8;
+
+// Targets per thread, warps per CTA and CTAs per cluster (source-row split).
+// A CTA's time is its pairs plus the lag tables it builds for them; the
+// device's is that times the CTAs an SM gets, stretched while the resident
+// warps times their independent targets are too few to cover the pipes'
+// latency.  KT: 1, 2, 4 (FP32), 1, 2 (FP64: registers).
+struct DirectTile { int KT, W, S, nchunk; };
+static DirectTile direct_tile(int nr, int nphi, bool f64)
+{
+    DirectTile best{1, 1, 1, 0};
+    double best_t = 1e300;
+    const double lag = f64 ? 60.0 : 45.0, pair = f64 ? 28.0 : 18.0;
+    for (int KT = 1; KT <= (f64 ? 2 : 4); KT *= 2)
+        for (int W = 1; W <= DMAXT / 32; ++W) {
+            const int TJ = 32 * W * KT;
+            if (W > 1 && 32 * (W - 1) * KT >= nphi) break;
+            const long long nchunk = (nphi + TJ - 1) / TJ;
+            for (int S = 1; S <= 8 && S <= nr; S *= 2) {
+                const double ctas = std::ceil((double)nr * nchunk * S / 152.0);   // per SM
+                const double work = std::ceil((double)nr / S) * nphi * (TJ * pair + lag + 2.0 * KT * W * 32 / DLT * 30);
+                const double hide = std::min(ctas * W, 32.0) * std::min(KT, 2);
+                const double t = ctas * work * std::max(1.0, (f64 ? 12.0 : 24.0) / hide);
+                if (t < best_t * 0.999) {
+                    best_t = t;
+                    best = {KT, W, S, (int)nchunk};
+                }
+            }
+        }
+    return best;
 }
 
 template <typename R>
@@ -151,12 +416,36 @@ cudaError_t launch_direct(int nr, int nphi, double r_in, double du, double G, co
 {
     (void)r_in;
     using P2 = typename pair_of<R>::type;
-    const int ncell = nr * nphi;
     const double dphi = 2.0 * M_PI / nphi;
-    k_direct<R><<<(ncell + DT - 1) / DT, DT, 0, s>>>(
-        nr, nphi, (R)G, sig_g, sig_d, Hg, Hd, (R)h_g, (R)h_d, tgt, phi, gr, gphi, (const P2 *)geo_i,
-        (const P2 *)geo_j, rcen, (R)(du * dphi), flag);
-    return cudaGetLastError();
+    if (nphi < kDirectRowMin) {
+        const int ncell = nr * nphi;
+        k_direct_short<R><<<(ncell + DT - 1) / DT, DT, 0, s>>>(
+            nr, nphi, (R)G, sig_g, sig_d, Hg, Hd, (R)h_g, (R)h_d, tgt, phi, gr, gphi, (const P2 *)geo_i,
+            (const P2 *)geo_j, rcen, (R)(du * dphi), flag);
+        return cudaGetLastError();
+    }
+    const DirectTile d = direct_tile(nr, nphi, sizeof(R) == 8);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)d.S;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nr * d.nchunk * d.S));
+    cfg.blockDim = dim3((unsigned)(32 * d.W));
+    cfg.dynamicSmemBytes = direct_smem<R>(32 * d.W, d.KT);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    auto go = [&](auto kern) {
+        return cudaLaunchKernelEx(&cfg, kern, nr, nphi, d.nchunk, (R)G, sig_g, sig_d, Hg, Hd, (R)h_g, (R)h_d, tgt, phi,
+                                  gr, gphi, (const P2 *)geo_i, (const P2 *)geo_j, rcen, (R)(du * dphi), flag);
+    };
+    cudaError_t e;
+    if (d.KT == 1) e = go(k_direct<R, 1>);
+    else if (d.KT == 2) e = go(k_direct<R, 2>);
+    else if constexpr (sizeof(R) == 4) e = go(k_direct<R, 4>);
+    else e = cudaErrorInvalidConfiguration;
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template cudaError_t launch_direct<float>(int, int, double, double, double, const float *, const float *,
