@@ -876,7 +876,7 @@ def run_semi(args):
             stages[name].append(float(v))
     mv_ms = statistics.mean(stages["semi_mv"])
     N = d.nphi // 2
-    table = 3 * N * d.nr * d.nr * 8
+    table = 3 * (N + 1) * d.nr * d.nr * 4
     mv_bytes = table + N * d.nr * 8 + 3 * N * d.nr * 8
     peak, peak_kind = measured_peaks()
     achieved = mv_bytes / (mv_ms * 1e-3) / 1e9

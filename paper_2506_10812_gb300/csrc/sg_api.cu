@@ -274,7 +274,7 @@ sg_status solve_t(sg_plan *pl, const void *sg_, const void *sd_, void *const out
                                sflag, pl->rows_fwd);
         if (e != cudaSuccess) return cuda_fail(pl, e, "row transform");
         if (ev) cudaEventRecord(pl->ev[1], s);
-        e = launch_semi_mv<R>(pl->sh, pl->tab, pl->oh, nr, nphi, pl->nsrc, mask, s);
+        e = launch_semi_mv<R>(pl->sh, pl->tab, pl->oh, nr, nphi, pl->nsrc, mask, s, !ev);
         if (e != cudaSuccess) return cuda_fail(pl, e, "radial products");
         if (ev) cudaEventRecord(pl->ev[2], s);
         RowOut ro{};
@@ -286,7 +286,7 @@ sg_status solve_t(sg_plan *pl, const void *sg_, const void *sd_, void *const out
             ++ro.n;
         }
         e = launch_rows_inv<R>(pl->oh, ro, nr, nphi, pl->tw_row, pl->twp_row, (const R *)pl->rcen, flag, s, 0, -1,
-                               pl->tm_rows ? &pl->tm_oh : nullptr, sflag, false, pl->rows_inv);
+                               pl->tm_rows ? &pl->tm_oh : nullptr, sflag, !ev, pl->rows_inv);
         if (e != cudaSuccess) return cuda_fail(pl, e, "inverse row transform");
         if (ev) cudaEventRecord(pl->ev[3], s);
     } else {
@@ -473,7 +473,7 @@ sg_status sg_plan_create(sg_plan **out, const sg_params *p, void *stream)
         const size_t need[] = {row_smem_bytes(p->nphi, row_rpc(p->nphi, pl->f64), pl->f64),
                                row_smem_bytes(p->nphi, row_rpc(p->nphi, true), true),
                                fft ? col_smem_bytes(p->nr, pl->nsrc, pl->f64) : semi_mv_smem(p->nr, pl->nsrc, pl->f64),
-                               fft ? tabcol_smem_bytes(pl->L, true) : 0};
+                               fft ? tabcol_smem_bytes(pl->L, true) : semi_table_smem(p->nphi, 0)};
         for (size_t b : need)
             if (b > (size_t)optin) return reject(SG_ERR_UNSUPPORTED, "grid too large for shared memory in this dtype");
     }
@@ -533,11 +533,9 @@ sg_status sg_plan_create(sg_plan **out, const sg_params *p, void *stream)
     SG_TRY(cudaMalloc((void **)&pl->ipart, (size_t)indirect_blocks(p->nphi) * 4 * sizeof(double)), "indirect sums");
     SG_TRY(cudaMemsetAsync(pl->flag, 0, sizeof(unsigned int), s), "flag");
     if (semi) {
-        SG_TRY(upload(&pl->tw_row64, twiddles<double>(p->nphi), s), "twiddles");
-        SG_TRY(upload(&pl->twp_row64, pass_twiddles<double>(p->nphi / 2), s), "twiddles");
         if (pl->f64) {
-            pl->tw_row = pl->tw_row64;
-            pl->twp_row = pl->twp_row64;
+            SG_TRY(upload(&pl->tw_row, twiddles<double>(p->nphi), s), "twiddles");
+            SG_TRY(upload(&pl->twp_row, pass_twiddles<double>(p->nphi / 2), s), "twiddles");
         } else {
             SG_TRY(upload(&pl->tw_row, twiddles<float>(p->nphi), s), "twiddles");
             SG_TRY(upload(&pl->twp_row, pass_twiddles<float>(p->nphi / 2), s), "twiddles");
@@ -558,10 +556,11 @@ sg_status sg_plan_create(sg_plan **out, const sg_params *p, void *stream)
         std::vector<double> rc(p->nr);
         for (int i = 0; i < p->nr; ++i) rc[i] = p->r_in * std::exp((i + 0.5) * pl->du);
         const double *hp[2] = {Hprof[0].data(), pl->nsrc == 2 ? Hprof[1].data() : nullptr};
+        const std::vector<double> twp = pass_twiddles<double>(p->nphi);
         SG_TRY(pl->f64 ? build_semi_tables<double>(p->nr, p->nphi, pl->nsrc, pl->du, pl->dphi, p->G, rc.data(), hp,
-                                                   pl->tab, pl->tw_row64, pl->twp_row64, s)
+                                                   pl->tab, twp.data(), twp.size(), s)
                        : build_semi_tables<float>(p->nr, p->nphi, pl->nsrc, pl->du, pl->dphi, p->G, rc.data(), hp,
-                                                  pl->tab, pl->tw_row64, pl->twp_row64, s),
+                                                  pl->tab, twp.data(), twp.size(), s),
                "semi-spectral table build");
     } else if (fft) {
         SG_TRY(upload(&pl->tw_row64, twiddles<double>(p->nphi), s), "twiddles");

@@ -135,19 +135,21 @@ cudaError_t launch_indirect(int nr, int nphi, int nsrc, const R *s0, const R *s1
                             double *out, cudaStream_t s);
 
 // Semi-spectral method (sg_semi.cu): tables of the phi-DFT of the exact pair
-// kernel for axisymmetric scale heights, [pair][component][nphi/2][nr][nr]
-// complex of type R (semi_table_bytes); rc_h, H_h[a]: host radial centres
-// and the source fluids' H profiles (FP64, nr each).  Synchronises `s`.
+// kernel for axisymmetric scale heights, [pair][component][nphi/2 + 1][nr][nr]
+// reals of type R (semi_table_bytes); rc_h, H_h[a]: host radial centres
+// and the source fluids' H profiles (FP64, nr each); twp_h: the per-pass FP64
+// twiddles of length nphi (twp_n doubles, host).  Synchronises `s`.
 size_t semi_table_bytes(int nr, int nphi, int nsrc, bool f64);
+size_t semi_table_smem(int nphi, int lgG);   // shared memory of a table CTA of 2^lgG rows
 template <typename R>
 cudaError_t build_semi_tables(int nr, int nphi, int nsrc, double du, double dphi, double G, const double *rc_h,
-                              const double *H_h[2], void *tab, const void *tw_row64, const void *twp_row64,
-                              cudaStream_t s);
+                              const double *H_h[2], void *tab, const double *twp_h, size_t twp_n, cudaStream_t s);
 // The per-mode matrix-vector products: row spectra sh ([nsrc][nphi/2][nr])
 // -> column output oh ([nsrc * 3][nphi/2][nr]) for the outputs in outmask.
+// pdl: programmatic dependent launch on the row transform before it.
 template <typename R>
 cudaError_t launch_semi_mv(const void *sh, const void *tab, void *oh, int nr, int nphi, int nsrc, uint32_t outmask,
-                           cudaStream_t s);
+                           cudaStream_t s, bool pdl = false);
 size_t semi_mv_smem(int nr, int nsrc, bool f64);
 cudaError_t set_semi_smem_limits(int max_optin);
 

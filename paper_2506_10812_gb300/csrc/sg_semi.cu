@@ -18,9 +18,12 @@
 // and 0 for the self cell; the direct path's pair terms, so the result is
 // the direct sum's.
 //
-// The plan stores W^ (FP64 kernel samples, FP64 row FFTs, rounded to the plan
-// dtype) as [pair][component][n_phi/2][n_r][n_r] complex, slot m = 0 packing
-// the real m = 0 and m = n_phi/2 matrices as re + i im like the row spectra.
+// With H = H(r) the samples are exactly even (W_Phi, W_r) or odd (W_phi) in
+// psi, so W^ is real, or imaginary for W_phi.  The plan stores one real number
+// per entry (FP64 samples and transforms, rounded to the plan dtype):
+// [pair][component][n_phi/2 + 1][n_r][n_r], W_phi's without its factor i.
+// The row spectra's slot m = 0 packs the real m = 0 and m = n_phi/2
+// coefficients as re + i im; its products take the planes m = 0 and n_phi/2.
 // The entries carry the conventions of the row transforms around them: the
 // forward rows multiply each source row by r_i', the inverse rows divide the
 // accelerations by r_i, and the inverse is unnormalised (1 / n_phi).  A solve
@@ -28,73 +31,138 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <vector>
+#include <algorithm>
 
 #include "sg_bessel.cuh"
 #include "sg_fft.cuh"
 #include "sg_internal.h"
+#include "sg_launch.h"
 #include "sg_mem.cuh"
 
 namespace sg {
 
 namespace {
 
-// Kernel samples of target rows i0 .. i0 + ci - 1 against every source row,
-// every lag: o_c[(il nr + i') nphi + dj], FP64.
-__global__ void __launch_bounds__(256)
-k_semi_eval(int nr, int nphi, int i0, int ci, const double *__restrict__ rc, const double *__restrict__ Ha,
-            const double *__restrict__ Hb, double du, double dphi, double G, double *__restrict__ o_phi,
-            double *__restrict__ o_r, double *__restrict__ o_a)
+// Lag tables in FP64: gi[i - i' + nr - 1] = (sinh^2(Delta/2), expm1(Delta)),
+// gj[dj] = (sin^2(psi/2), sin psi).
+__global__ void k_semi_geometry(int nr, int nphi, double du, double2 *gi, double2 *gj)
 {
-    __shared__ BesselWeights bw;
-    bessel_weights_init(bw);
-    __syncthreads();
-    const double inv_sqrt_pi = 0.56418958354775628695;
-    const size_t n = (size_t)ci * nr * nphi;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int row = (int)(idx / nphi), dj = (int)(idx - (size_t)row * nphi);
-        const int il = row / nr, ip = row - il * nr, i = i0 + il;
-        double vP = 0.0, vR = 0.0, vA = 0.0;
-        if (!(i == ip && dj == 0)) {
-            const double r = rc[i], rp = rc[ip];
-            const double Dl = (i - ip) * du;
-            const double sh = sinh(0.5 * Dl);
-            const double sp = sinpi((double)dj / nphi);               // sin(psi / 2)
-            const double sp2 = sp * sp;
-            const double s2 = 4.0 * r * rp * (sh * sh + sp2);
-            const double H2 = 0.5 * (Ha[ip] * Ha[ip] + Hb[i] * Hb[i]);
-            const double X = s2 / (8.0 * H2);
-            double k0e, Dx;
-            k0e_D_f64(X, bw, k0e, Dx);
-            const double invH = 1.0 / sqrt(H2);
-            const double mu = G * rp * rp * du * dphi;
-            const double f = -mu * Dx * (0.125 * inv_sqrt_pi) * invH * invH * invH;
-            // row transforms: sources enter times r_i', accelerations leave divided by
-            // r_i, the inverse is unnormalised
-            const double acc = r / (rp * nphi), pot = 1.0 / (rp * nphi);
-            vR = f * rp * (expm1(Dl) + 2.0 * sp2) * acc;
-            vA = f * rp * sinpi(2.0 * dj / nphi) * acc;
-            vP = -mu * k0e * (0.5 * inv_sqrt_pi) * invH * pot;
+    const int n = max(2 * nr - 1, nphi);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        if (q < 2 * nr - 1) {
+            const double D = (q - (nr - 1)) * du, sh = sinh(0.5 * D);
+            gi[q] = make_double2(sh * sh, expm1(D));
         }
-        o_phi[idx] = vP;
-        o_r[idx] = vR;
-        o_a[idx] = vA;
+        if (q < nphi) {
+            const double sp = sinpi((double)q / nphi);
+            gj[q] = make_double2(sp * sp, sinpi(2.0 * q / nphi));
+        }
     }
 }
 
-// Packed row spectra of the chunk ([nphi/2][ci nr], FP64) -> the table rows
-// i0 .. i0 + ci - 1 of one (pair, component): tab[(m nr + i) nr + i'].
-template <typename R>
-__global__ void __launch_bounds__(256)
-k_semi_pack(const double2 *__restrict__ spec, cplx<R> *__restrict__ tab, int nr, int N, int i0, int ci)
+// Tables of one (source, target) pair of fluids: a CTA owns G source rows i'
+// of one target row i (blockIdx.y), n_phi / 16 threads each.  It samples the
+// three components for dj = 0 .. n_phi/2, mirrors them, transforms the row in
+// registers and writes the real coefficients, G consecutive entries at a
+// time; nothing passes through device memory in between.
+//
+// FP64 arithmetic bounds it (2 lanes per clock and SM), so the work is cut:
+// half the samples by symmetry; one short polynomial per Bessel function (as in
+// the direct sum, lengths in units of sqrt(r r')); and, for an FP32 plan, one
+// complex transform for the three components, (W_Phi + W_phi) + i W_r, whose
+// parts are separable because W_Phi and W_r are even and W_phi odd.  An FP64
+// plan transforms W_Phi by itself (PASS 1) and W_r + W_phi (PASS 2), so that no
+// component takes on the rounding of a larger one.  128 x 256 gas + dust:
+// 15.5 -> 2.3 ms for a plan, a solve and the release (12.5 ms of it was sampling by
+// branch, 2.0 ms twelve real transforms).
+template <typename R, int PASS>
+__global__ void __launch_bounds__(512)
+k_semi_table(int nr, int nphi, int lgG, const double2 *__restrict__ gi, const double2 *__restrict__ gj,
+             const double *__restrict__ rc, const double *__restrict__ Ha, const double *__restrict__ Hb, double scale,
+             R *__restrict__ tab, const double2 *__restrict__ tw)
 {
-    const size_t rows = (size_t)ci * nr, n = (size_t)N * rows;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t m = idx / rows, k = idx - m * rows;
-        const double2 v = spec[blk(m, k, rows)];
-        tab[(m * nr + i0) * nr + k] = mkc<cplx<R>>((R)v.x, (R)v.y);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int T = nphi >> 4, N = nphi >> 1, G = 1 << lgG, PL = padded_len(nphi);
+    double2 *buf = reinterpret_cast<double2 *>(smem_raw);
+    double *sc = reinterpret_cast<double *>(buf + (size_t)G * PL);      // per row: eta, prefactor
+    const int g = threadIdx.x / T, t = threadIdx.x - g * T;
+    const int i = blockIdx.y, ip0 = blockIdx.x * G, ip = ip0 + g;
+    for (int k = threadIdx.x; k < G; k += blockDim.x) {
+        const double r = rc[i], p = rc[ip0 + k], q2 = 1.0 / (r * p), ha = Ha[ip0 + k], hb = Hb[i];
+        sc[2 * k] = 0.5 * (ha * ha + hb * hb) * q2;
+        sc[2 * k + 1] = scale * p * sqrt(q2);
+    }
+    __syncthreads();
+    double2 *xb = buf + (size_t)g * PL;
+    const double2 li = gi[i - ip + nr - 1];
+    {
+        const double inv_sqrt_pi = 0.56418958354775628695;
+        const double eta = sc[2 * g], A = sc[2 * g + 1], y = rsqrt(eta), ix = 0.5 / eta;
+        const double cP = A * (0.5 * inv_sqrt_pi) * y, cF = A * (0.25 * inv_sqrt_pi) * y;
+#pragma unroll 1
+        for (int dj = t; dj <= N; dj += T) {
+            const double2 lj = gj[dj];
+            const double sg = li.x + lj.x, X = sg * ix;                 // sigma = 4 sg
+            double P = 0.0, F = 0.0;
+            if (!(i == ip && dj == 0)) {                                // self cell excluded
+                const double i1 = rsqrt(sg), isg = i1 * i1;
+                if (X >= 16.0) {
+                    double S0, Q;
+                    bessel_tail(2.0 * eta * isg, S0, Q);
+                    P = 0.5 * A * i1 * S0;
+                    F = 0.125 * A * i1 * isg * Q;
+                } else if (bessel_in_table(X)) {
+                    double k0e, E;
+                    bessel_table(X, k0e, E);
+                    P = cP * k0e;
+                    F = cF * isg * E;
+                } else {                                                // X < 2^-20, or not a number
+                    double k0e, D;
+                    k0e_D_series(X, k0e, D);
+                    P = cP * k0e;
+                    F = cF * isg * (D * X);
+                }
+            }
+            const double vR = F * (li.y + 2.0 * lj.x), vA = dj == N ? 0.0 : F * lj.y;
+            double2 z, zm;                                              // at dj and at -dj
+            if constexpr (PASS == 0) {
+                z = make_double2(P + vA, vR);
+                zm = make_double2(P - vA, vR);
+            } else if constexpr (PASS == 1) {
+                z = zm = make_double2(P, 0.0);
+            } else {
+                z = make_double2(vR + vA, 0.0);
+                zm = make_double2(vR - vA, 0.0);
+            }
+            xb[pidx(dj)] = z;
+            if (dj > 0 && dj < N) xb[pidx(nphi - dj)] = zm;
+        }
+    }
+    __syncthreads();
+    double2 v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = xb[pidx(t + T * e)];
+    fft_reg<true>(v, nphi, T, t, xb, tw);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) xb[pidx(t + T * e)] = v[e];
+    __syncthreads();
+    const size_t plane = (size_t)nr * nr, comp = (size_t)(N + 1) * plane;
+    for (int idx = threadIdx.x; idx < (N + 1) << lgG; idx += blockDim.x) {
+        const int gg = idx & (G - 1), m = idx >> lgG;
+        const double2 Z = buf[(size_t)gg * PL + pidx(m)], Zm = buf[(size_t)gg * PL + pidx((nphi - m) & (nphi - 1))];
+        R *o = tab + m * plane + (size_t)i * nr + ip0 + gg;
+        const double even = 0.5 * (Z.x + Zm.x), odd = 0.5 * (Z.y - Zm.y);
+        if constexpr (PASS == 0) {
+            o[0] = (R)even;
+            o[comp] = (R)(0.5 * (Z.y + Zm.y));
+            o[2 * comp] = (R)odd;
+        } else if constexpr (PASS == 1) {
+            o[0] = (R)even;
+        } else {
+            o[comp] = (R)even;
+            o[2 * comp] = (R)odd;
+        }
     }
 }
 
@@ -105,64 +173,72 @@ struct SemiOut {
 // One CTA: mode m, 32 target rows, one requested output.  The source spectra
 // of column m wait in shared memory; each warp runs 4 target rows, its lanes
 // striding the source rows of each table row (each table entry is read once,
-// streaming).  Slot m = 0 multiplies re by re and im by im (two real
-// matrices, the m = 0 and m = nphi/2 modes).
+// streaming).  Slot m = 0 multiplies re by plane 0 and im by plane n_phi/2.
+// The stream of the tables bounds it: one real number per entry is half the
+// bytes of a complex table: 512 x 1024 gas 1.61 GB in 246 us (0.97 of the
+// measured HBM bandwidth), 3.23 GB in 537 us before.
+template <typename R> struct vec_of;
+template <> struct vec_of<float> { using type = float4; };
+template <> struct vec_of<double> { using type = double2; };
+
 template <typename R, int NS>
 __global__ void __launch_bounds__(256)
-k_semi_mv(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<R> *__restrict__ oh, int nr,
+k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__restrict__ oh, int nr,
           int N, const __grid_constant__ SemiOut q)
 {
     using C = cplx<R>;
+    using V = typename vec_of<R>::type;
+    constexpr int W = sizeof(V) / sizeof(R);              // entries per 16-byte load
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *ss = reinterpret_cast<C *>(smem_raw);
     const int m = blockIdx.x, z = blockIdx.z, b = q.b[z], c = q.c[z];
+    griddep_launch();
+    griddep_wait();                                       // the row spectra are complete from here on
     for (int k = threadIdx.x; k < NS * nr; k += blockDim.x) {
         const int a = k / nr, ip = k - a * nr;
-        ss[k] = sh[(size_t)a * N * nr + blk(m, ip, nr)];
+        ss[k] = ld_cg_hint(sh + (size_t)a * N * nr + blk(m, ip, nr), l2_evict_last());
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int ib = blockIdx.y * 32 + w * 4;
-    const bool packed0 = m == 0;
+    const size_t plane = (size_t)nr * nr;
     R ar[4] = {0, 0, 0, 0}, ai[4] = {0, 0, 0, 0};
+    // nr is a power of two >= 8, so a warp's four rows are all in the grid
+    const size_t r0 = (size_t)ib * nr, r1 = r0 + nr, r2 = r1 + nr, r3 = r2 + nr;
 #pragma unroll 1
     for (int a = 0; a < NS; ++a) {
-        const C *T = tab + ((size_t)((a * NS + b) * 3 + c) * N + m) * nr * nr;
+        const R *T = tab + ((size_t)((a * NS + b) * 3 + c) * (N + 1) + m) * plane;
         const C *sa = ss + a * nr;
-        if constexpr (sizeof(R) == 4) {
-            // two complex per lane per step (16-byte loads; nr is even); four
-            // steps of four rows in flight per thread
+        if (m != 0) {
 #pragma unroll 4
-            for (int ip = 2 * lane; ip < nr; ip += 64) {
-                const float4 s = *reinterpret_cast<const float4 *>(sa + ip);
+            for (int ip = W * lane; ip < nr; ip += 32 * W) {
+                const V t[4] = {__ldcs(reinterpret_cast<const V *>(T + r0 + ip)),
+                                __ldcs(reinterpret_cast<const V *>(T + r1 + ip)),
+                                __ldcs(reinterpret_cast<const V *>(T + r2 + ip)),
+                                __ldcs(reinterpret_cast<const V *>(T + r3 + ip))};
+                C s[W];
+#pragma unroll
+                for (int x = 0; x < W; x += 16 / sizeof(C))
+                    *reinterpret_cast<float4 *>(&s[x]) = *reinterpret_cast<const float4 *>(sa + ip + x);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    if (ib + k >= nr) break;
-                    const float4 t = __ldcs(reinterpret_cast<const float4 *>(T + (size_t)(ib + k) * nr + ip));
-                    if (packed0) {
-                        ar[k] = fmaf(t.x, s.x, fmaf(t.z, s.z, ar[k]));
-                        ai[k] = fmaf(t.y, s.y, fmaf(t.w, s.w, ai[k]));
-                    } else {
-                        ar[k] = fmaf(t.x, s.x, fmaf(-t.y, s.y, fmaf(t.z, s.z, fmaf(-t.w, s.w, ar[k]))));
-                        ai[k] = fmaf(t.x, s.y, fmaf(t.y, s.x, fmaf(t.z, s.w, fmaf(t.w, s.z, ai[k]))));
+                    const R *tk = reinterpret_cast<const R *>(&t[k]);
+#pragma unroll
+                    for (int x = 0; x < W; ++x) {
+                        ar[k] = fma(tk[x], s[x].x, ar[k]);
+                        ai[k] = fma(tk[x], s[x].y, ai[k]);
                     }
                 }
             }
         } else {
-#pragma unroll 2
+            const R *TN = T + (size_t)N * plane;
+            const size_t rk[4] = {r0, r1, r2, r3};
             for (int ip = lane; ip < nr; ip += 32) {
                 const C s = sa[ip];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    if (ib + k >= nr) break;
-                    const C t = T[(size_t)(ib + k) * nr + ip];
-                    if (packed0) {
-                        ar[k] = fma(t.x, s.x, ar[k]);
-                        ai[k] = fma(t.y, s.y, ai[k]);
-                    } else {
-                        ar[k] = fma(t.x, s.x, fma(-t.y, s.y, ar[k]));
-                        ai[k] = fma(t.x, s.y, fma(t.y, s.x, ai[k]));
-                    }
+                    ar[k] = fma(T[rk[k] + ip], s.x, ar[k]);
+                    ai[k] = fma(TN[rk[k] + ip], s.y, ai[k]);
                 }
             }
         }
@@ -175,7 +251,7 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<
             ai[k] += __shfl_xor_sync(0xffffffffu, ai[k], o);
         }
     }
-    if (lane < 4 && ib + lane < nr) {
+    if (lane < 4) {
         R xr = ar[0], xi = ai[0];
 #pragma unroll
         for (int k = 1; k < 4; ++k)
@@ -183,71 +259,73 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<
                 xr = ar[k];
                 xi = ai[k];
             }
-        oh[(size_t)(b * 3 + c) * N * nr + blk(m, ib + lane, nr)] = mkc<C>(xr, xi);
+        C v = mkc<C>(xr, xi);
+        if (c == 2 && m != 0) v = cmul_i(v);              // planes 0 and n_phi/2 of the odd component are zero
+        oh[(size_t)(b * 3 + c) * N * nr + blk(m, ib + lane, nr)] = v;
     }
 }
-
-int grid_for(size_t n) { return (int)((n + 255) / 256 < 152 * 32 ? (n + 255) / 256 : 152 * 32); }
 
 }  // namespace
 
 size_t semi_table_bytes(int nr, int nphi, int nsrc, bool f64)
 {
-    return (size_t)nsrc * nsrc * 3 * (nphi / 2) * (size_t)nr * nr * (f64 ? 16 : 8);
+    return (size_t)nsrc * nsrc * 3 * (nphi / 2 + 1) * (size_t)nr * nr * (f64 ? 8 : 4);
 }
 
 template <typename R>
 cudaError_t build_semi_tables(int nr, int nphi, int nsrc, double du, double dphi, double G, const double *rc_h,
-                              const double *H_h[2], void *tab, const void *tw_row64, const void *twp_row64,
-                              cudaStream_t s)
+                              const double *H_h[2], void *tab, const double *twp_h, size_t twp_n, cudaStream_t s)
 {
-    const int N = nphi / 2;
-    // chunk of target rows: 3 component samples + one spectrum, ~512 MB of FP64 scratch
-    const size_t per_row = (size_t)nr * nphi * 8 * 4;
-    int ci = 1;
-    while (ci < nr && (size_t)(2 * ci) * per_row <= ((size_t)512 << 20)) ci *= 2;
-    double *rc = nullptr, *H = nullptr, *eval = nullptr;
-    void *spec = nullptr;
-    const size_t chunk = (size_t)ci * nr * nphi;
-    cudaError_t e = cudaMalloc((void **)&rc, nr * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&H, 2 * (size_t)nr * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&eval, 3 * chunk * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&spec, chunk * sizeof(double));   // [N][ci nr] complex
+    // scratch: the two lag tables, the transform's twiddles, the radii and the profiles
+    const size_t ngi = 2 * (size_t)(2 * nr), ngj = 2 * (size_t)nphi;
+    double *scr = nullptr;
+    cudaError_t e = cudaMalloc((void **)&scr, (ngi + ngj + twp_n + 3 * (size_t)nr) * sizeof(double));
+    if (e != cudaSuccess) return e;
+    double2 *gi = (double2 *)scr, *gj = (double2 *)(scr + ngi);
+    double *tw = scr + ngi + ngj, *rc = tw + twp_n, *H = rc + nr;
+    e = cudaMemcpyAsync(tw, twp_h, twp_n * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(rc, rc_h, nr * sizeof(double), cudaMemcpyHostToDevice, s);
     for (int a = 0; a < nsrc && e == cudaSuccess; ++a)
         e = cudaMemcpyAsync(H + (size_t)a * nr, H_h[a], nr * sizeof(double), cudaMemcpyHostToDevice, s);
-    const size_t one = (size_t)N * nr * nr;   // entries of one (pair, component) table
+    if (e == cudaSuccess) {
+        k_semi_geometry<<<(std::max(2 * nr, nphi) + 255) / 256, 256, 0, s>>>(nr, nphi, du, gi, gj);
+        e = cudaGetLastError();
+    }
+    // rows per CTA: 256 threads (512 for the longest rows) and at most the radial cells
+    const int T = nphi / 16;
+    int lgG = 0;
+    while ((T << (lgG + 1)) <= 256 && (1 << (lgG + 1)) <= nr) ++lgG;
+    const size_t smem = semi_table_smem(nphi, lgG);
+    const dim3 grid(nr >> lgG, nr), block(T << lgG);
+    const double scale = -G * du * dphi / nphi;
     for (int a = 0; a < nsrc && e == cudaSuccess; ++a)
-        for (int b = 0; b < nsrc && e == cudaSuccess; ++b)
-            for (int i0 = 0; i0 < nr && e == cudaSuccess; i0 += ci) {
-                double *o[3] = {eval, eval + chunk, eval + 2 * chunk};
-                k_semi_eval<<<grid_for(chunk), 256, 0, s>>>(nr, nphi, i0, ci, rc, H + (size_t)a * nr,
-                                                           H + (size_t)b * nr, du, dphi, G, o[0], o[1], o[2]);
-                e = cudaGetLastError();
-                for (int c = 0; c < 3 && e == cudaSuccess; ++c) {
-                    e = launch_rows_fwd<double>(o[c], nullptr, 1, spec, ci * nr, nphi, tw_row64, twp_row64, nullptr,
-                                                false, s);
-                    if (e != cudaSuccess) break;
-                    cplx<R> *dst = reinterpret_cast<cplx<R> *>(tab) + (size_t)((a * nsrc + b) * 3 + c) * one;
-                    k_semi_pack<R><<<grid_for((size_t)N * ci * nr), 256, 0, s>>>((const double2 *)spec, dst, nr, N,
-                                                                                 i0, ci);
-                    e = cudaGetLastError();
-                }
+        for (int b = 0; b < nsrc && e == cudaSuccess; ++b) {
+            R *dst = (R *)tab + (size_t)(a * nsrc + b) * 3 * (nphi / 2 + 1) * nr * nr;
+            auto go = [&](auto kern) {
+                kern<<<grid, block, smem, s>>>(nr, nphi, lgG, gi, gj, rc, H + (size_t)a * nr, H + (size_t)b * nr, scale, dst,
+                                               (const double2 *)tw);
+            };
+            if constexpr (sizeof(R) == 4) {
+                go(k_semi_table<R, 0>);
+            } else {
+                go(k_semi_table<R, 1>);
+                go(k_semi_table<R, 2>);
             }
+            e = cudaGetLastError();
+        }
     cudaError_t e2 = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = e2;
-    cudaFree(rc);
-    cudaFree(H);
-    cudaFree(eval);
-    cudaFree(spec);
+    cudaFree(scr);
     return e;
 }
+
+size_t semi_table_smem(int nphi, int lgG) { return ((size_t)padded_len(nphi) * 16 + 16) << lgG; }
 
 size_t semi_mv_smem(int nr, int nsrc, bool f64) { return (size_t)nsrc * nr * (f64 ? 16 : 8); }
 
 template <typename R>
 cudaError_t launch_semi_mv(const void *sh, const void *tab, void *oh, int nr, int nphi, int nsrc, uint32_t outmask,
-                           cudaStream_t s)
+                           cudaStream_t s, bool pdl)
 {
     SemiOut q{};
     int nz = 0;
@@ -262,17 +340,18 @@ cudaError_t launch_semi_mv(const void *sh, const void *tab, void *oh, int nr, in
     const dim3 grid(N, (nr + 31) / 32, nz);
     const size_t smem = semi_mv_smem(nr, nsrc, sizeof(R) == 8);
     using C = cplx<R>;
-    if (nsrc == 1)
-        k_semi_mv<R, 1><<<grid, 256, smem, s>>>((const C *)sh, (const C *)tab, (C *)oh, nr, N, q);
-    else
-        k_semi_mv<R, 2><<<grid, 256, smem, s>>>((const C *)sh, (const C *)tab, (C *)oh, nr, N, q);
-    return cudaGetLastError();
+    const int threads = nr >= 32 ? 256 : nr * 8;          // 4 target rows a warp
+    const cudaError_t e = launch_ex(nsrc == 1 ? k_semi_mv<R, 1> : k_semi_mv<R, 2>, grid, dim3(threads), smem, s, pdl,
+                                    (const C *)sh, (const R *)tab, (C *)oh, nr, N, q);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t set_semi_smem_limits(int max_optin)
 {
-    const void *fns[] = {(const void *)k_semi_mv<float, 1>, (const void *)k_semi_mv<float, 2>,
-                         (const void *)k_semi_mv<double, 1>, (const void *)k_semi_mv<double, 2>};
+    const void *fns[] = {(const void *)k_semi_mv<float, 1>,       (const void *)k_semi_mv<float, 2>,
+                         (const void *)k_semi_mv<double, 1>,      (const void *)k_semi_mv<double, 2>,
+                         (const void *)k_semi_table<float, 0>,    (const void *)k_semi_table<double, 1>,
+                         (const void *)k_semi_table<double, 2>};
     for (const void *f : fns) {
         const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
         if (e != cudaSuccess) return e;
@@ -281,10 +360,12 @@ cudaError_t set_semi_smem_limits(int max_optin)
 }
 
 template cudaError_t build_semi_tables<float>(int, int, int, double, double, double, const double *,
-                                              const double *[2], void *, const void *, const void *, cudaStream_t);
+                                              const double *[2], void *, const double *, size_t, cudaStream_t);
 template cudaError_t build_semi_tables<double>(int, int, int, double, double, double, const double *,
-                                               const double *[2], void *, const void *, const void *, cudaStream_t);
-template cudaError_t launch_semi_mv<float>(const void *, const void *, void *, int, int, int, uint32_t, cudaStream_t);
-template cudaError_t launch_semi_mv<double>(const void *, const void *, void *, int, int, int, uint32_t, cudaStream_t);
+                                               const double *[2], void *, const double *, size_t, cudaStream_t);
+template cudaError_t launch_semi_mv<float>(const void *, const void *, void *, int, int, int, uint32_t, cudaStream_t,
+                                           bool);
+template cudaError_t launch_semi_mv<double>(const void *, const void *, void *, int, int, int, uint32_t, cudaStream_t,
+                                            bool);
 
 }  // namespace sg
