@@ -530,7 +530,8 @@ sg_status sg_plan_create(sg_plan **out, const sg_params *p, void *stream)
     if (pl->f64) SG_TRY(upload(&pl->rcen, centres<double>(p->nr, p->r_in, pl->du), s), "centres");
     else SG_TRY(upload(&pl->rcen, centres<float>(p->nr, p->r_in, pl->du), s), "centres");
     SG_TRY(cudaMalloc((void **)&pl->flag, sizeof(unsigned int)), "flag");
-    SG_TRY(cudaMalloc((void **)&pl->ipart, (size_t)indirect_blocks(p->nphi) * 4 * sizeof(double)), "indirect sums");
+    SG_TRY(cudaMalloc((void **)&pl->ipart, indirect_doubles(p->nphi) * sizeof(double)), "indirect sums");
+    SG_TRY(launch_indirect_angles(p->nphi, pl->ipart, s), "indirect sums");
     SG_TRY(cudaMemsetAsync(pl->flag, 0, sizeof(unsigned int), s), "flag");
     if (semi) {
         if (pl->f64) {

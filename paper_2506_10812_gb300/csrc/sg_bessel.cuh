@@ -205,4 +205,23 @@ __device__ __forceinline__ void bessel_tail(double z, double &S0, double &Q)
     }
 }
 
+// (K0e, D) at any x: table, tail or series (FP64; 10 to 14 multiply-adds a
+// function in place of the quadrature above).
+__device__ __forceinline__ void k0e_D_short(double x, double &k0e, double &D)
+{
+    if (x >= 16.0) {
+        double S0, Q;
+        const double y = rsqrt(x), z = y * y, s = 1.2533141373155002512 * y;     // sqrt(pi / 2)
+        bessel_tail(z, S0, Q);
+        k0e = s * S0;
+        D = 0.5 * s * z * Q;
+    } else if (bessel_in_table(x)) {
+        double E;
+        bessel_table(x, k0e, E);
+        D = E / x;
+    } else {
+        k0e_D_series(x, k0e, D);                   // x < 2^-20, or not a number
+    }
+}
+
 }  // namespace sg

@@ -126,12 +126,14 @@ cudaError_t launch_rows_inv(const void *oh, const RowOut &o, int nr, int nphi, c
                             int nrows_run = -1, const CUtensorMap *tm = nullptr, unsigned int *tflag = nullptr,
                             bool pdl = false, int tile_rows = 2);
 
-// Indirect term (App. E): out[2 a + {0, 1}] = (A_a, B_a) in FP64; partial
-// holds indirect_blocks(nphi) x 4 doubles.
-int indirect_blocks(int nphi);
+// Indirect term (App. E): out[2 a + {0, 1}] = (A_a, B_a) in FP64; buf holds
+// indirect_doubles(nphi) doubles, its table laid out once by
+// launch_indirect_angles.
+size_t indirect_doubles(int nphi);
+cudaError_t launch_indirect_angles(int nphi, double *buf, cudaStream_t s);
 template <typename R>
 cudaError_t launch_indirect(int nr, int nphi, int nsrc, const R *s0, const R *s1, const R *H0, const R *H1,
-                            double h0, double h1, const R *rcen, double G, double du, double dphi, double *partial,
+                            double h0, double h1, const R *rcen, double G, double du, double dphi, double *buf,
                             double *out, cudaStream_t s);
 
 // Semi-spectral method (sg_semi.cu): tables of the phi-DFT of the exact pair
@@ -178,7 +180,7 @@ struct sg_plan {
     void *rcen = nullptr, *geo_i = nullptr, *geo_j = nullptr;
     void *Hg = nullptr, *Hd = nullptr;
     unsigned int *flag = nullptr;         // bit 1: non-finite output, bit 2: staging timeout
-    double *ipart = nullptr;              // indirect-term partial sums
+    double *ipart = nullptr;              // indirect term: partial sums and the azimuths' cosines and sines
     void *stage = nullptr;                // sg_solve_host: [2 inputs + 6 outputs][cells]
     int engine = 0;                       // column-pass engine (SG_ENGINE_*)
     uint32_t *atab = nullptr;             // its A-fragment table (tensor-core engines)
