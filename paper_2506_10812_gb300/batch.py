@@ -8,7 +8,7 @@ import ctypes
 import torch
 
 from . import _native as N
-from .plan import _OUT_KEYS
+from .plan import _OUT_KEYS, _current_stream, _on_device
 
 
 class Batch:
@@ -64,12 +64,12 @@ class Batch:
         self._h = h
 
     def _stream(self):
-        return ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        return _current_stream(self.device)
 
     def solve(self):
         """Every disc, one graph launch (asynchronous)."""
-        with torch.cuda.device(self.device):
-            N.check(self._lib.sg_batch_solve(self._h, self._stream()), what="sg_batch_solve", batch_handle=self._h)
+        st = _on_device(self.device, self._lib.sg_batch_solve, self._h, self._stream())
+        N.check(st, what="sg_batch_solve", batch_handle=self._h)
 
     def solve_loop(self):
         """The per-disc baseline: sg_solve on every plan in turn."""

@@ -16,8 +16,28 @@ from . import _native as N
 _OUT_KEYS = ("phi_g", "gr_g", "gphi_g", "phi_d", "gr_d", "gphi_d")
 
 
+# The stream handle alone: building a Stream object costs 2 us, as much as a
+# launch, and a small disc's solve is bound by the calling thread.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _current_stream(device):
+    """Handle of torch's current stream on ``device`` (an int, for ctypes)."""
+    if _raw_stream is not None:
+        return _raw_stream(device.index)
+    return torch.cuda.current_stream(device).cuda_stream
+
+
+def _on_device(device, fn, *args):
+    """fn(*args) with ``device`` current (the guard object only where another one is)."""
+    if torch.cuda.current_device() == device.index:
+        return fn(*args)
+    with torch.cuda.device(device):
+        return fn(*args)
+
+
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 class Plan:
@@ -43,6 +63,7 @@ class Plan:
             raise ValueError("dtype must be torch.float32 or torch.float64")
         self.dtype = dtype
         self.nr, self.nphi = int(nr), int(nphi)
+        self._shape = torch.Size((max(self.nr, 0), max(self.nphi, 0)))
         self.r_in, self.r_out = float(r_in), float(r_out)
         self.h_g = float(h_g) if h_g is not None else 0.0
         self.h_d = float(h_d) if h_d else 0.0
@@ -73,9 +94,12 @@ class Plan:
 
     # ------------------------------------------------------------------
     def _stream(self):
-        return ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        return _current_stream(self.device)
 
     def _check(self, t, name):
+        if (isinstance(t, torch.Tensor) and t.shape == self._shape and t.dtype is self.dtype and
+                t.device == self.device and t.is_contiguous()):
+            return t
         if not isinstance(t, torch.Tensor):
             raise TypeError(f"{name} must be a torch tensor")
         if t.device != self.device:
@@ -116,27 +140,25 @@ class Plan:
         for k, v in res.items():
             self._check(v, k)
         ptrs = [_ptr(res.get(k)) for k in _OUT_KEYS]
-        with torch.cuda.device(self.device):
-            st = self._lib.sg_solve(self._h, _ptr(sigma_g), _ptr(sigma_d), *ptrs, self._stream())
+        st = _on_device(self.device, self._lib.sg_solve, self._h, _ptr(sigma_g), _ptr(sigma_d), *ptrs,
+                        self._stream())
         N.check(st, self._h, "sg_solve")
         return res
 
     def potential(self, sigma_g, sigma_d=None):
         sigma_g, sigma_d = self._inputs(sigma_g, sigma_d)
         res = self._alloc(self._keys(("phi",)))
-        with torch.cuda.device(self.device):
-            st = self._lib.sg_potential(self._h, _ptr(sigma_g), _ptr(sigma_d), _ptr(res.get("phi_g")),
-                                        _ptr(res.get("phi_d")), self._stream())
+        st = _on_device(self.device, self._lib.sg_potential, self._h, _ptr(sigma_g), _ptr(sigma_d),
+                        _ptr(res.get("phi_g")), _ptr(res.get("phi_d")), self._stream())
         N.check(st, self._h, "sg_potential")
         return res
 
     def accel(self, sigma_g, sigma_d=None):
         sigma_g, sigma_d = self._inputs(sigma_g, sigma_d)
         res = self._alloc(self._keys(("gr", "gphi")))
-        with torch.cuda.device(self.device):
-            st = self._lib.sg_accel(self._h, _ptr(sigma_g), _ptr(sigma_d), _ptr(res.get("gr_g")),
-                                    _ptr(res.get("gphi_g")), _ptr(res.get("gr_d")), _ptr(res.get("gphi_d")),
-                                    self._stream())
+        st = _on_device(self.device, self._lib.sg_accel, self._h, _ptr(sigma_g), _ptr(sigma_d),
+                        _ptr(res.get("gr_g")), _ptr(res.get("gphi_g")), _ptr(res.get("gr_d")),
+                        _ptr(res.get("gphi_d")), self._stream())
         N.check(st, self._h, "sg_accel")
         return res
 
@@ -145,8 +167,8 @@ class Plan:
         [[A_g, B_g], ([A_d, B_d])] on the plan's device."""
         sigma_g, sigma_d = self._inputs(sigma_g, sigma_d)
         out = torch.empty((2 if self.bifluid else 1, 2), dtype=torch.float64, device=self.device)
-        with torch.cuda.device(self.device):
-            st = self._lib.sg_indirect(self._h, _ptr(sigma_g), _ptr(sigma_d), _ptr(out), self._stream())
+        st = _on_device(self.device, self._lib.sg_indirect, self._h, _ptr(sigma_g), _ptr(sigma_d), _ptr(out),
+                        self._stream())
         N.check(st, self._h, "sg_indirect")
         return out
 
