@@ -66,8 +66,9 @@ std::vector<R> twiddles(int M)
     return v;
 }
 
-// Per-pass Stockham twiddles of a length-L transform (layout in sg_fft.cuh):
-// for the pass with stride Ns and radix R, W_{Ns R}^{r k} at (r - 1) Ns + k.
+// Per-pass Stockham twiddles of a length-L transform (layouts in sg_fft.cuh):
+// FP32, for the pass with stride Ns and radix R, W_{Ns R}^{r k} at (r - 1) Ns + k;
+// FP64, the roots of fft_f64.
 template <typename R>
 std::vector<R> pass_twiddles(int L)
 {
@@ -80,6 +81,26 @@ std::vector<R> pass_twiddles(int L)
                 v.push_back((R)(-std::sin(a)));
             }
     };
+    // FP64: the roots of fft_f64's levels, w^p exp(-2 pi i j / 16), as {p, j}
+    static const int r16[8][2] = {{8, 0}, {4, 0}, {2, 0}, {2, 2}, {1, 0}, {1, 1}, {1, 2}, {1, 3}};
+    static const int r8[4][2] = {{4, 0}, {2, 0}, {1, 0}, {1, 2}}, r4[2][2] = {{2, 0}, {1, 0}}, r2[1][2] = {{1, 0}};
+    auto put64 = [&](int Ns, int Rad) {
+        const int (*rows)[2] = Rad == 16 ? r16 : Rad == 8 ? r8 : Rad == 4 ? r4 : r2;
+        for (int q = 0; q < Rad / 2; ++q)
+            for (int k = 0; k < Ns; ++k) {
+                // exp(-2 pi i (p k / (Ns Rad) + j / 16)) as cosine and tangent, the fraction exact
+                const double a = 2.0 * M_PI * ((double)(rows[q][0] * k) / ((double)Ns * Rad) + rows[q][1] / 16.0);
+                v.push_back((R)std::cos(a));
+                v.push_back((R)(-std::tan(a)));
+            }
+    };
+    if (sizeof(R) == 8) {
+        int Ns = 16;
+        for (; Ns * 16 <= L; Ns *= 16) put64(Ns, 16);
+        if (Ns < L) put64(Ns, L / Ns);
+        if (v.empty()) v.assign(2, (R)0);
+        return v;
+    }
     int Ns = 16;
     while (Ns * 16 <= L) {
         put(Ns, 16);

@@ -14,7 +14,8 @@
 // pass with stride Ns and radix R reads W_{Ns R}^{r k} = exp(-2 pi i r k / (Ns R))
 // at (r - 1) Ns + k, so the threads of a warp (consecutive k) read
 // consecutive entries; the passes' segments follow one another (Ns = 16,
-// 256, ... for the radix-16 passes, then the final pass).
+// 256, ... for the radix-16 passes, then the final pass).  FP64 transforms take
+// another set of roots per pass (fft_f64).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -50,6 +51,17 @@ template <typename T> __device__ __forceinline__ T cfma(T a, T b, T acc)
     acc.x += a.x * b.x - a.y * b.y;
     acc.y += a.x * b.y + a.y * b.x;
     return acc;
+}
+// acc + a * b and acc + a * conj(b) as four multiply-adds (FP64, where every
+// instruction counts; the compiler may not reassociate the form above into it.
+// FP32 columns of length 4096 measured 0.6 % slower with it.)
+__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 acc)
+{
+    return mkc<double2>(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
+}
+__device__ __forceinline__ double2 cfmac(double2 a, double2 b, double2 acc)
+{
+    return mkc<double2>(fma(a.x, b.x, fma(a.y, b.y, acc.x)), fma(a.y, b.x, fma(-a.x, b.y, acc.y)));
 }
 template <bool FWD, typename T> __device__ __forceinline__ T twmul(T a, T w)
 {
@@ -297,6 +309,184 @@ __device__ __forceinline__ void final_pass(T (&v)[16], int t, int T_, int Ns, co
     }
 }
 
+// ---------------------------------------------------------------- FP64
+// FP64 instructions bound these transforms (two lanes per clock and SM), so
+// they are written for the fewest: every radix-2 butterfly takes its root with
+// it.  A root is held as (c, t), w = c (1 + i t) (cosine and tangent, after Linzer and
+// Feig's multiply-add transforms): (u, v) = b (1 + i t) takes two multiply-adds, a + c (u, v) and
+// a - c (u, v) two each, six instructions and two roundings per value where a
+// complex product and two sums are eight and three.  (t may be as large as
+// 1.6e16, at a right angle: c t is the sine to rounding, and what the sum
+// b.x - t b.y then drops of b.x is c b.x < 1e-16 |b|.)  A
+// radix-16 pass is four such levels, the input twiddles w^r folded into them:
+// level by level the roots are w^8; w^4 (and -i w^4); w^2 W8^k; w W16^k (k = 0,
+// 1, and so on; the upper half of each level is -i times the lower), so that a
+// pass reads 8 roots from its table, not 15, and is 192 instructions instead
+// of 228; the first pass, with constants, 148 instead of 168.
+// Table (pass_twiddles<double>): per pass of stride Ns, w = exp(-2 pi i k / (Ns R)),
+// rows of Ns roots: radix 16: w^8, w^4, w^2, w^2 W8, w, w W16, w W8, w W16^3;
+// radix 8: w^4, w^2, w, w W8; radix 4: w^2, w; radix 2: w.
+// (a, b) <- (a + w b, a - w b), w conjugated for the inverse transform
+template <bool FWD> __device__ __forceinline__ void bfly(double2 &a, double2 &b, double2 w)
+{
+    const double t = FWD ? w.y : -w.y;
+    const double u = fma(-t, b.y, b.x), v = fma(t, b.x, b.y);
+    b = make_double2(fma(-w.x, u, a.x), fma(-w.x, v, a.y));
+    a = make_double2(fma(w.x, u, a.x), fma(w.x, v, a.y));
+}
+// the same with the root -i w
+template <bool FWD> __device__ __forceinline__ void bfly_mi(double2 &a, double2 &b, double2 w)
+{
+    b = FWD ? cmul_mi(b) : cmul_i(b);
+    bfly<FWD>(a, b, w);
+}
+__device__ __forceinline__ void bfly_1(double2 &a, double2 &b)
+{
+    const double2 t = a;
+    a = cadd(t, b);
+    b = csub(t, b);
+}
+template <bool FWD> __device__ __forceinline__ void bfly_1mi(double2 &a, double2 &b)   // root -i
+{
+    const double2 t = a, u = FWD ? cmul_mi(b) : cmul_i(b);
+    a = cadd(t, u);
+    b = csub(t, u);
+}
+// bit-reversed registers to natural order (renaming only)
+__device__ __forceinline__ void unreverse16(double2 (&v)[16])
+{
+    double2 b[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) b[i] = v[i];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[((i & 1) << 3) | ((i & 2) << 1) | ((i & 4) >> 1) | (i >> 3)] = b[i];
+}
+// first pass (all w = 1); HALF: v[8..15] are zero
+template <bool FWD, bool HALF> __device__ __forceinline__ void dft16_f64(double2 (&v)[16])
+{
+    const double2 W8 = make_double2(SG_C8, -1.0), W16 = make_double2(SG_C16, -0.41421356237309504880),
+                  W163 = make_double2(SG_S16, -2.41421356237309504880);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        if constexpr (HALF) v[r + 8] = v[r];
+        else bfly_1(v[r], v[r + 8]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        bfly_1(v[r], v[r + 4]);
+        bfly_1mi<FWD>(v[r + 8], v[r + 12]);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        bfly_1(v[r], v[r + 2]);
+        bfly_1mi<FWD>(v[r + 4], v[r + 6]);
+        bfly<FWD>(v[r + 8], v[r + 10], W8);
+        bfly_mi<FWD>(v[r + 12], v[r + 14], W8);
+    }
+    bfly_1(v[0], v[1]);
+    bfly_1mi<FWD>(v[2], v[3]);
+    bfly<FWD>(v[4], v[5], W8);
+    bfly_mi<FWD>(v[6], v[7], W8);
+    bfly<FWD>(v[8], v[9], W16);
+    bfly_mi<FWD>(v[10], v[11], W16);
+    bfly<FWD>(v[12], v[13], W163);
+    bfly_mi<FWD>(v[14], v[15], W163);
+    unreverse16(v);
+}
+// a later radix-16 pass; tp: its table row 0 at this thread's k
+template <bool FWD> __device__ __forceinline__ void pass16_f64(double2 (&v)[16], const double2 *__restrict__ tp, int Ns)
+{
+    const double2 w8 = __ldg(tp), w4 = __ldg(tp + Ns), w2 = __ldg(tp + 2 * Ns), w2a = __ldg(tp + 3 * Ns);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) bfly<FWD>(v[r], v[r + 8], w8);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        bfly<FWD>(v[r], v[r + 4], w4);
+        bfly_mi<FWD>(v[r + 8], v[r + 12], w4);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        bfly<FWD>(v[r], v[r + 2], w2);
+        bfly_mi<FWD>(v[r + 4], v[r + 6], w2);
+        bfly<FWD>(v[r + 8], v[r + 10], w2a);
+        bfly_mi<FWD>(v[r + 12], v[r + 14], w2a);
+    }
+    const double2 w = __ldg(tp + 4 * Ns), wa = __ldg(tp + 5 * Ns), wb = __ldg(tp + 6 * Ns), wc = __ldg(tp + 7 * Ns);
+    bfly<FWD>(v[0], v[1], w);
+    bfly_mi<FWD>(v[2], v[3], w);
+    bfly<FWD>(v[4], v[5], wb);
+    bfly_mi<FWD>(v[6], v[7], wb);
+    bfly<FWD>(v[8], v[9], wa);
+    bfly_mi<FWD>(v[10], v[11], wa);
+    bfly<FWD>(v[12], v[13], wc);
+    bfly_mi<FWD>(v[14], v[15], wc);
+    unreverse16(v);
+}
+// final pass of radix RL: butterfly q combines registers q + r Q
+template <bool FWD, int RL>
+__device__ __forceinline__ void final_f64(double2 (&v)[16], int t, int T_, int Ns, const double2 *__restrict__ tp0)
+{
+    constexpr int Q = 16 / RL;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const double2 *tp = tp0 + ((t + T_ * q) & (Ns - 1));
+        double2 *x = v + q;                           // element r at x[r Q]
+        if constexpr (RL == 2) {
+            bfly<FWD>(x[0], x[Q], __ldg(tp));
+        } else if constexpr (RL == 4) {
+            const double2 w2 = __ldg(tp), w = __ldg(tp + Ns);
+            bfly<FWD>(x[0], x[2 * Q], w2);
+            bfly<FWD>(x[Q], x[3 * Q], w2);
+            bfly<FWD>(x[0], x[Q], w);
+            bfly_mi<FWD>(x[2 * Q], x[3 * Q], w);
+            const double2 y = x[Q];                   // order 0, 2, 1, 3
+            x[Q] = x[2 * Q];
+            x[2 * Q] = y;
+        } else {
+            const double2 w4 = __ldg(tp), w2 = __ldg(tp + Ns), w = __ldg(tp + 2 * Ns), wa = __ldg(tp + 3 * Ns);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) bfly<FWD>(x[r * Q], x[(r + 4) * Q], w4);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                bfly<FWD>(x[r * Q], x[(r + 2) * Q], w2);
+                bfly_mi<FWD>(x[(r + 4) * Q], x[(r + 6) * Q], w2);
+            }
+            bfly<FWD>(x[0], x[Q], w);
+            bfly_mi<FWD>(x[2 * Q], x[3 * Q], w);
+            bfly<FWD>(x[4 * Q], x[5 * Q], wa);
+            bfly_mi<FWD>(x[6 * Q], x[7 * Q], wa);
+            double2 y = x[Q];                         // order 0, 4, 2, 6, 1, 5, 3, 7
+            x[Q] = x[4 * Q];
+            x[4 * Q] = y;
+            y = x[3 * Q];
+            x[3 * Q] = x[6 * Q];
+            x[6 * Q] = y;
+        }
+    }
+}
+// Full length-L FP64 transform, layout and contract of fft_reg below.
+template <bool FWD, bool HALF = false>
+__device__ __forceinline__ void fft_f64(double2 (&v)[16], int L, int T_, int t, double2 *xb,
+                                        const double2 *__restrict__ twp)
+{
+    dft16_f64<FWD, HALF>(v);
+    if (L == 16) return;
+    int Ns = 16;
+    const double2 *tp = twp;
+    exchange16(v, t, T_, 1, xb);
+    while (Ns * 16 <= L) {
+        pass16_f64<FWD>(v, tp + (t & (Ns - 1)), Ns);
+        tp += 8 * Ns;
+        if (Ns * 16 == L) return;
+        exchange16(v, t, T_, Ns, xb);
+        Ns *= 16;
+    }
+    const int RL = L / Ns;
+    if (RL == 8) final_f64<FWD, 8>(v, t, T_, Ns, tp);
+    else if (RL == 4) final_f64<FWD, 4>(v, t, T_, Ns, tp);
+    else final_f64<FWD, 2>(v, t, T_, Ns, tp);
+}
+
 // Full length-L transform (L = 16 T_, power of two) of the strided register
 // layout v[e] = x[t + T_ e]; result X[t + T_ e] in v[e].  Forward: X[k] =
 // sum x[n] exp(-2 pi i n k / L); inverse: the same with +i (unnormalised).
@@ -306,6 +496,10 @@ __device__ __forceinline__ void final_pass(T (&v)[16], int t, int T_, int Ns, co
 template <bool FWD, typename T>
 __device__ __forceinline__ void fft_reg(T (&v)[16], int L, int T_, int t, T *xb, const T *__restrict__ twp)
 {
+    if constexpr (sizeof(T) == 16) {
+        fft_f64<FWD>(v, L, T_, t, xb, twp);
+        return;
+    }
     dft16<FWD>(v);                              // pass Ns = 1: no twiddles
     if (L == 16) return;
     int Ns = 16;
@@ -473,14 +667,15 @@ __device__ __forceinline__ void fft_ct(T (&v)[16], int t, T *xb, const T *__rest
     fft_ct_pass<FWD, L, 16>(v, t, xb, twp, b, d16);
 }
 
-// Compile-time length when LC > 0, runtime length L otherwise (the
-// butterfly policy d16 and the zero-half pruning HALF apply to the
-// compile-time lengths).
+// Compile-time length when LC > 0 (FP32), runtime length L otherwise (the
+// butterfly policy d16 applies to the compile-time lengths, the zero-half
+// pruning HALF to those and to FP64).
 template <bool FWD, int LC, bool HALF = false, typename T, typename D16 = RegDft16<FWD>>
 __device__ __forceinline__ void fft_any(T (&v)[16], int L, int T_, int t, T *xb, const T *__restrict__ twp,
                                         D16 &&d16 = D16{})
 {
-    if constexpr (LC > 0) fft_ct<FWD, LC, HALF>(v, t, xb, twp, d16);
+    if constexpr (sizeof(T) == 16) fft_f64<FWD, HALF>(v, L, T_, t, xb, twp);
+    else if constexpr (LC > 0) fft_ct<FWD, LC, HALF>(v, t, xb, twp, d16);
     else fft_reg<FWD>(v, L, T_, t, xb, twp);
 }
 

@@ -149,20 +149,22 @@ using ColsKernel = void (*)(const cplx<R> *, const cplx<R> *, cplx<R> *, int, in
 template <typename R>
 ColsKernel<R> cols_kernel_all(int nsrc, int L)
 {
-    const bool f64 = sizeof(R) == 8;
-    if (nsrc == 1) {
-        if (!f64 && L == 4096) return k_cols<R, 1, 4096, false>;
-        if (!f64 && L == 2048) return k_cols<R, 1, 2048, false>;
-        if (!f64 && L == 1024) return k_cols<R, 1, 1024, false>;
-        if (!f64 && L == 512) return k_cols<R, 1, 512, false>;
-        if (!f64 && L == 256) return k_cols<R, 1, 256, false>;
-        return k_cols<R, 1, 0, false>;
+    if constexpr (sizeof(R) == 4) {
+        if (nsrc == 1) {
+            if (L == 4096) return k_cols<R, 1, 4096, false>;
+            if (L == 2048) return k_cols<R, 1, 2048, false>;
+            if (L == 1024) return k_cols<R, 1, 1024, false>;
+            if (L == 512) return k_cols<R, 1, 512, false>;
+            if (L == 256) return k_cols<R, 1, 256, false>;
+        } else {
+            if (L == 4096) return k_cols<R, 2, 4096, false>;
+            if (L == 2048) return k_cols<R, 2, 2048, false>;
+            if (L == 1024) return k_cols<R, 2, 1024, false>;
+            if (L == 512) return k_cols<R, 2, 512, false>;
+            if (L == 256) return k_cols<R, 2, 256, false>;
+        }
     }
-    if (!f64 && L == 4096) return k_cols<R, 2, 4096, false>;
-    if (!f64 && L == 2048) return k_cols<R, 2, 2048, false>;
-    if (!f64 && L == 1024) return k_cols<R, 2, 1024, false>;
-    if (!f64 && L == 512) return k_cols<R, 2, 512, false>;
-    if (!f64 && L == 256) return k_cols<R, 2, 256, false>;
+    if (nsrc == 1) return k_cols<R, 1, 0, false>;
     return k_cols<R, 2, 0, false>;
 }
 

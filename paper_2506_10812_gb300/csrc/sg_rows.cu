@@ -259,7 +259,7 @@ template <int NC, int NR> int fwd_resident_ctas()
 // the row mean before the transform.
 // NC > 0: compile-time row transform length (nphi / 2).
 template <typename R, int NC>
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 1024, 1)   // FP64: at most 512 (row_rpc)
 k_rows_fwd(const R *__restrict__ x0, const R *__restrict__ x1, cplx<R> *__restrict__ xh, int nrows,
            int nphi_rt, int rpc, const cplx<R> *__restrict__ tw, const cplx<R> *__restrict__ twp,
            const R *__restrict__ rscale, int dc, int row0)
@@ -279,13 +279,16 @@ k_rows_fwd(const R *__restrict__ x0, const R *__restrict__ x1, cplx<R> *__restri
     const C *xr = reinterpret_cast<const C *>((a == 0 ? x0 : x1) + (size_t)(i0 + g) * nphi);
     C *xb = sm + g * padded_len(N);
     C v[16];
-    const R sc = rscale ? rscale[i0 + g] : (R)1;
+    // FP64 (bound by its instructions): half the row's scale, which is the R2C
+    // step's factor 1/2, and scale and mean in one multiply-add
+    constexpr bool F64 = sizeof(R) == 8;
+    const R sc = (F64 ? (R)0.5 : (R)1) * (rscale ? rscale[i0 + g] : (R)1);
 #pragma unroll
     for (int e = 0; e < 16; ++e) {                        // z[n] = x[2n] + i x[2n+1]
         const C z = xr[t + T * e];
-        v[e] = mkc<C>(z.x * sc, z.y * sc);
+        v[e] = F64 ? z : mkc<C>(z.x * sc, z.y * sc);
     }
-    R mean = 0;
+    R mean = 0;                                           // of the scaled row
     if (dc) {
         R s = 0;
 #pragma unroll
@@ -301,12 +304,19 @@ k_rows_fwd(const R *__restrict__ x0, const R *__restrict__ x1, cplx<R> *__restri
             const int w0 = (g * T) >> 5, nw = T >> 5;
             for (int w = 0; w < nw; ++w) s += red[w0 + w];
         }
-        mean = s / (R)nphi;
+        mean = F64 ? s * sc / (R)nphi : s / (R)nphi;
+        if constexpr (!F64) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = mkc<C>(v[e].x - mean, v[e].y - mean);
+            for (int e = 0; e < 16; ++e) v[e] = mkc<C>(v[e].x - mean, v[e].y - mean);
+        }
+    }
+    if constexpr (F64) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = mkc<C>(fma(v[e].x, sc, -mean), fma(v[e].y, sc, -mean));
     }
     fft_any<true, NC>(v, N, T, t, xb, twp);
     // X[k] = E[k] + W^k O[k], E = (Z[k] + Z*[N-k]) / 2, O = (Z[k] - Z*[N-k]) / 2i
+    // (FP64: Z is of the halved row)
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; ++e) xb[pidx(t + T * e)] = v[e];
@@ -323,12 +333,17 @@ k_rows_fwd(const R *__restrict__ x0, const R *__restrict__ x1, cplx<R> *__restri
         const C Z = v[e];
         if (e == 0 && t == 0) {
             // (X[0], X[nphi/2]) packed; the mean only enters X[0]
-            v[e] = mkc<C>(Z.x + Z.y + mean * (R)nphi, Z.x - Z.y);
+            const R two = F64 ? (R)2 : (R)1;
+            v[e] = mkc<C>(two * (Z.x + Z.y + mean * (R)nphi), two * (Z.x - Z.y));
         } else {
             const C Zc = cconj(xb[FAST ? zc0 - e * (T + T / 16) : pidx(N - k)]);
-            const C E = cscale(cadd(Z, Zc), (R)0.5);
-            const C O = cscale(cmul_mi(csub(Z, Zc)), (R)0.5);
-            v[e] = cadd(E, cmul(O, __ldg(&tw[k])));
+            if constexpr (F64) {
+                v[e] = cfma(cmul_mi(csub(Z, Zc)), __ldg(&tw[k]), cadd(Z, Zc));
+            } else {
+                const C E = cscale(cadd(Z, Zc), (R)0.5);
+                const C O = cscale(cmul_mi(csub(Z, Zc)), (R)0.5);
+                v[e] = cadd(E, cmul(O, __ldg(&tw[k])));
+            }
         }
     }
     // write through a [N][rpc] tile: rpc consecutive rows of each column (x BW columns)
@@ -400,16 +415,20 @@ cudaError_t launch_rows_fwd(const R *x0, const R *x1, int nsrc, void *xh, int nr
             x0, x1, (cplx<R> *)xh, nrows, nphi, rpc, (const cplx<R> *)tw_row, (const cplx<R> *)twp_row, rscale,
             dc ? 1 : 0, row0);
     };
-    if (!f64 && nphi == 4096) go(k_rows_fwd<R, 2048>);
-    else if (!f64 && nphi == 2048) go(k_rows_fwd<R, 1024>);
-    else go(k_rows_fwd<R, 0>);
+    if constexpr (sizeof(R) == 4) {
+        if (nphi == 4096) go(k_rows_fwd<R, 2048>);
+        else if (nphi == 2048) go(k_rows_fwd<R, 1024>);
+        else go(k_rows_fwd<R, 0>);
+    } else {
+        go(k_rows_fwd<R, 0>);
+    }
     return cudaGetLastError();
 }
 
 
 // ------------------------------------------------------- row C2R + epilogue
 template <typename R, int NC>
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(sizeof(R) == 8 ? 512 : 1024, 1)   // FP64: at most 512 (row_rpc)
 k_rows_inv(const cplx<R> *__restrict__ oh, const __grid_constant__ RowOut o, int nrows, int nphi_rt, int rpc,
            const cplx<R> *__restrict__ tw, const cplx<R> *__restrict__ twp, const R *__restrict__ rcen,
            unsigned int *flag, int row0)
@@ -475,7 +494,8 @@ k_rows_inv(const cplx<R> *__restrict__ oh, const __grid_constant__ RowOut o, int
             v[e] = mkc<C>(X.x + X.y, X.x - X.y);
         } else {
             const C Xc = cconj(sm[FAST ? xc0 - 4 * T * e : tile_idx_g<C>(N - k, g, lg)]);
-            v[e] = cadd(cadd(X, Xc), cmul_i(cmulc(csub(X, Xc), __ldg(&tw[k]))));
+            if constexpr (sizeof(R) == 8) v[e] = cfmac(cmul_i(csub(X, Xc)), __ldg(&tw[k]), cadd(X, Xc));
+            else v[e] = cadd(cadd(X, Xc), cmul_i(cmulc(csub(X, Xc), __ldg(&tw[k]))));
         }
     }
     // the transform's exchange buffer overlays the tile; fft_reg
@@ -640,9 +660,13 @@ cudaError_t launch_rows_inv(const void *oh, const RowOut &o, int nr, int nphi, c
                         (const cplx<R> *)oh, o, nr, nphi, rpc, (const cplx<R> *)tw_row, (const cplx<R> *)twp_row, rcen,
                         flag, row0);
     };
-    if (!f64 && nphi == 4096) go(k_rows_inv<R, 2048>);
-    else if (!f64 && nphi == 2048) go(k_rows_inv<R, 1024>);
-    else go(k_rows_inv<R, 0>);
+    if constexpr (sizeof(R) == 4) {
+        if (nphi == 4096) go(k_rows_inv<R, 2048>);
+        else if (nphi == 2048) go(k_rows_inv<R, 1024>);
+        else go(k_rows_inv<R, 0>);
+    } else {
+        go(k_rows_inv<R, 0>);
+    }
     return err != cudaSuccess ? err : cudaGetLastError();
 }
 
