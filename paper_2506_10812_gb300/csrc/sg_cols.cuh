@@ -73,6 +73,7 @@ __device__ __noinline__ void col0_output(const cplx<R> *__restrict__ sh, const c
         }
         __syncthreads();                           // before the next transform rewrites the buffer
     }
+    griddep_launch();
     fft_any<false, LC>(acc, L, T, t, xb, tw);
     C *o = oh + (size_t)q * N * nr;
 #pragma unroll
@@ -102,6 +103,20 @@ constexpr int cols_max_threads(int ns, bool f64, int lc, bool st) { return cols_
 constexpr int cols_min_blocks(int ns, bool f64, int lc, bool st)
 {
     return cols_tight(ns, f64, lc, st) ? 768 / (lc / 16) : 1;
+}
+
+// One CTA per (column, output) instead of one per column: NS + 1 transforms in
+// series instead of NS + the outputs, for the forward transforms repeated by every
+// output.  Worth it while the chip is idle otherwise: a column CTA is a chain of
+// latencies, so as long as all CTAs of the split launch are resident at once
+// (FP32: 128 registers, 512 threads per SM) it is the chain that counts.  FP64
+// instructions take a sub-partition 64 cycles a warp, so there the line is
+// one warp per sub-partition.
+inline bool cols_split(int N, int T, int nq, bool f64)
+{
+    if (nq < 2) return false;
+    const long long ctas = (long long)N * nq;
+    return f64 ? ctas * ((T + 31) / 32) <= 152 * 4 : ctas * (T < 32 ? 32 : T) <= 152 * 512;
 }
 
 // Columns m >= 1 of a plan that stages kernel spectra per step (ST = 1):
@@ -142,7 +157,9 @@ __device__ __forceinline__ void cols_pair_steps(const cplx<R> *__restrict__ sh, 
     if (q >= 0) issue(q);                          // lands while the forward FFTs run
     griddep_wait();                                // the row spectra are complete from here on
     C spec[NS][16];
-#pragma unroll
+    // one copy of the transform for both sources (a small grid's CTA runs its
+    // code once, and fetching it is part of its time), the results moved to their registers
+#pragma unroll 1
     for (int a = 0; a < NS; ++a) {
         C v[16];
         const uint64_t pf = l2_evict_first();
@@ -155,7 +172,10 @@ __device__ __forceinline__ void cols_pair_steps(const cplx<R> *__restrict__ sh, 
         // transform's first barrier: the column is dead
         if (discard) l2_discard_range(sh + (size_t)a * N * nr + blk(m, 0, nr), (size_t)nr * sizeof(C), t, T);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) spec[a][e] = v[e];
+        for (int e = 0; e < 16; ++e) {
+            if (NS == 1 || a == 0) spec[0][e] = v[e];
+            if (NS == 2) spec[NS - 1][e] = v[e];
+        }
     }
     for (int s = 0; q >= 0; ++s) {
         const int b = q / 3, c = q % 3;
@@ -180,7 +200,9 @@ __device__ __forceinline__ void cols_pair_steps(const cplx<R> *__restrict__ sh, 
             fence_proxy_async();
             issue(qn);
         }
+        if (qn < 0 && s == 0) griddep_launch();
         fft_any<false, LC>(v, L, T, t, xb, tw, eng.template d16<false>());
+        if (qn < 0 && s > 0) griddep_launch();
         C *o = oh + (size_t)(b * 3 + c) * N * nr;
         const uint64_t pl = l2_evict_last();
 #pragma unroll
@@ -189,9 +211,18 @@ __device__ __forceinline__ void cols_pair_steps(const cplx<R> *__restrict__ sh, 
     }
 }
 
+// When the inverse rows may launch (griddep_launch): late, before a CTA's last
+// stores (before its last inverse transform if that is its only one).  Resident
+// early, they only wait, but they take the places that the columns have left
+// free, which are not spread evenly over the SMs, and run there: letting them
+// launch from the first instruction cost 256 x 512 gas + dust 16.8 us instead of 12.5,
+// 512 x 1024 26.5 / 23.4, 1024 x 2048 gas 36.0 / 34.8, 2048 x 4096 126.9 / 125.6.
+//
 // Column pass: one CTA per requested output of column 0, then one CTA per
 // column m >= 1 (LC: compile-time column length, 0 for any; ST: staging as
-// above; outmask holds the requested outputs of this plan's fluids only).
+// above; outmask holds the requested outputs of this plan's fluids only).  A
+// split launch (gridDim.y = the number of outputs) has one CTA per column and output,
+// each with its own forward transforms (cols_split).
 template <typename R, int NS, int LC, bool ST>
 __global__ void __launch_bounds__(cols_max_threads(NS, sizeof(R) == 8, LC, ST),
                                   cols_min_blocks(NS, sizeof(R) == 8, LC, ST))
@@ -205,13 +236,24 @@ k_cols(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<R> 
     const int L = 2 * nr, T = L >> 4, H = nr, P = tab_pitch(nr);
     C *xb = reinterpret_cast<C *>(smem_raw + 16);
     C *tb = reinterpret_cast<C *>(smem_raw + 16 + align16((size_t)padded_len(L) * sizeof(C)));
-    const int t = threadIdx.x, nq = __popc(outmask), m = (int)blockIdx.x - nq + 1;
-    griddep_launch();                     // the inverse rows may set up once every column CTA runs
+    const int t = threadIdx.x;
+    const bool split = gridDim.y > 1;
+    int m, y;                             // column, and the output of a column-0 or split CTA (its rank in outmask)
+    if (split) {
+        m = blockIdx.x;
+        y = blockIdx.y;
+    } else {
+        m = (int)blockIdx.x - __popc(outmask) + 1;
+        y = blockIdx.x;
+    }
+    if (split || m < 1) {
+        for (; y > 0; --y) outmask &= outmask - 1;
+        outmask &= 0u - outmask;
+    }
     static_assert(!ST || sizeof(R) == 4, "per-step staging is FP32 only");
     constexpr bool PAIR = ST;
     if (m < 1) {
-        // column 0: CTA i computes the i-th requested output
-        col0_output<R, NS, LC>(sh, tab, oh, nr, N, (int)__fns(outmask, 0, (int)blockIdx.x + 1), tw, xb);
+        col0_output<R, NS, LC>(sh, tab, oh, nr, N, __ffs((int)outmask) - 1, tw, xb);
         return;
     }
     if constexpr (PAIR) {
@@ -294,7 +336,10 @@ k_cols(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<R> 
                 }
                 v[e] = acc;
             }
+            const bool last = (outmask >> (3 * b + c + 1)) == 0, one = (outmask & (outmask - 1)) == 0;
+            if (last && one) griddep_launch();
             fft_any<false, LC>(v, L, T, t, xb, tw);
+            if (last && !one) griddep_launch();
             C *o = oh + (size_t)(b * 3 + c) * N * nr;
             const uint64_t pl = l2_evict_last();
 #pragma unroll

@@ -177,14 +177,16 @@ cudaError_t launch_cols(const void *sh, const void *tab, void *oh, int nr, int n
     const int N = nphi / 2, T = (2 * nr) / 16;
     const bool steps = cols_staging_steps(nr, nsrc, f64, staging);
     const size_t smem = col_smem_bytes(nr, nsrc, f64, steps ? 1 : 0);
-    const int grid = (ncols > 0 && ncols < N ? ncols : N) - 1 + __builtin_popcount(outmask);
-    // whole 128-byte lines per source column (column 0 is read by every
-    // output's CTA and never discarded)
-    const bool dc = discard && BW == 1 && ((size_t)nr * 2 * sizeof(R)) % 128 == 0 && ((uintptr_t)sh & 127u) == 0;
+    const int nq = __builtin_popcount(outmask);
+    const bool split = ncols <= 0 && cols_split(N, T, nq, f64);
+    const dim3 grid = split ? dim3(N, nq) : dim3((ncols > 0 && ncols < N ? ncols : N) - 1 + nq);
+    // whole 128-byte lines per source column (a column read by every output's
+    // CTA, column 0 or a split launch's, is not discarded)
+    const bool dc = discard && !split && BW == 1 && ((size_t)nr * 2 * sizeof(R)) % 128 == 0 && ((uintptr_t)sh & 127u) == 0;
     ColsKernel<R> kern;
     if constexpr (sizeof(R) == 4) kern = steps ? cols_kernel_steps(nsrc, 2 * nr) : cols_kernel_all<R>(nsrc, 2 * nr);
     else kern = cols_kernel_all<R>(nsrc, 2 * nr);
-    const cudaError_t err = launch_ex(kern, dim3(grid), dim3(T), smem, s, pdl, (const cplx<R> *)sh,
+    const cudaError_t err = launch_ex(kern, grid, dim3(T), smem, s, pdl, (const cplx<R> *)sh,
                                       (const cplx<R> *)tab, (cplx<R> *)oh, nr, N, outmask,
                                       (const cplx<R> *)tw_col, flag, dc ? 1 : 0);
     return err != cudaSuccess ? err : cudaGetLastError();

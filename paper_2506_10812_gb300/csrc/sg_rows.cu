@@ -131,12 +131,12 @@ template <int NC, int NR>
 __global__ void __launch_bounds__(rows_tma_threads(NC, NR), rows_tma_min_blocks(NC, NR, 1024))
 k_rows_fwd_tma(const float *__restrict__ x0, const float *__restrict__ x1, const __grid_constant__ CUtensorMap tm,
                const float2 *__restrict__ tw, const float2 *__restrict__ twp, const float *__restrict__ rscale,
-               int dc, unsigned int *tflag, int row0, int ahead)
+               int dc, unsigned int *tflag, int row0, int ahead, int late)
 {
     static_assert(NR == 2 || NR == 4, "the tensor-copy row transforms take 2 or 4 rows per CTA");
     constexpr int N = NC, T = N / 16, NW = NR * T / 32, PLS = row_pitch_tma(N, NR), XS = T + T / 16;
     extern __shared__ __align__(1024) unsigned char smem_tma[];
-    griddep_launch();                     // the column pass may set up once every row CTA runs
+    if (!late) griddep_launch();          // the column pass may set up once every row CTA runs
     float *red = reinterpret_cast<float *>(smem_tma + 64);              // NW x NR partial sums
     float2 *reg = reinterpret_cast<float2 *>(smem_tma + kRowHdr);
     if (smem_u32(reg) & 127u) {                                         // TMA alignment (never expected)
@@ -214,6 +214,7 @@ k_rows_fwd_tma(const float *__restrict__ x0, const float *__restrict__ x1, const
             v[e] = cadd(E, cmul(O, tw_step<e>(w0)));
         }
     });
+    if (late) griddep_launch();
     __syncthreads();                                      // the tile overwrites the exchange buffers
     float2 *tl = reg + NR * t + g;
 #pragma unroll
@@ -391,10 +392,15 @@ cudaError_t launch_rows_fwd(const R *x0, const R *x1, int nsrc, void *xh, int nr
         // whole tiles, each starting on a 16-byte boundary of the map's rows
         if (tm && aligned && rows_tma_eligible(nrows, nphi, false) && nrows_run % NR == 0 && row0 % NR == 0) {
             const dim3 gt(nrows_run / NR, nsrc);
+            // fewer CTAs than SMs: column CTAs that launch at once would pack the
+            // idle SMs, so they launch when the rows are about to leave (512 x 1024
+            // gas 17.0 -> 13.6 us); with every SM busy early is better (2048 x 4096 gas
+            // 129.0 against 130.4, 1024 x 2048 34.8 against 35.3)
+            const int late = (long long)gt.x * gt.y <= 152;
             auto go = [&](auto kern, int N, int ahead) {
                 kern<<<gt, NR * N / 16, row_tma_smem_bytes(N, NR), s>>>(x0, x1, *tm, (const float2 *)tw_row,
                                                                         (const float2 *)twp_row, rscale, dc ? 1 : 0,
-                                                                        tflag, row0, ahead);
+                                                                        tflag, row0, ahead, late);
             };
             if (NR == 2) {
                 if (nphi == 4096) go(k_rows_fwd_tma<2048, 2>, 2048, fwd_resident_ctas<2048, 2>());

@@ -192,7 +192,6 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *ss = reinterpret_cast<C *>(smem_raw);
     const int m = blockIdx.x, z = blockIdx.z, b = q.b[z], c = q.c[z];
-    griddep_launch();
     griddep_wait();                                       // the row spectra are complete from here on
     for (int k = threadIdx.x; k < NS * nr; k += blockDim.x) {
         const int a = k / nr, ip = k - a * nr;
@@ -243,6 +242,7 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__
             }
         }
     }
+    griddep_launch();                                     // the inverse rows, late (as in the column pass)
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
 #pragma unroll
