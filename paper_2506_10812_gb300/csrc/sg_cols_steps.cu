@@ -14,6 +14,8 @@ ColsKernelF32 cols_kernel_steps(int nsrc, int L)
         if (L == 1024) return k_cols<float, 1, 1024, true>;
         if (L == 512) return k_cols<float, 1, 512, true>;
         if (L == 256) return k_cols<float, 1, 256, true>;
+        if (L == 128) return k_cols<float, 1, 128, true>;
+        if (L == 64) return k_cols<float, 1, 64, true>;
         return k_cols<float, 1, 0, true>;
     }
     if (L == 4096) return k_cols<float, 2, 4096, true>;
@@ -21,13 +23,15 @@ ColsKernelF32 cols_kernel_steps(int nsrc, int L)
     if (L == 1024) return k_cols<float, 2, 1024, true>;
     if (L == 512) return k_cols<float, 2, 512, true>;
     if (L == 256) return k_cols<float, 2, 256, true>;
+    if (L == 128) return k_cols<float, 2, 128, true>;
+    if (L == 64) return k_cols<float, 2, 64, true>;
     return k_cols<float, 2, 0, true>;
 }
 
 cudaError_t set_cols_steps_smem_limits(int max_optin)
 {
     for (int nsrc = 1; nsrc <= 2; ++nsrc)
-        for (int L : {0, 256, 512, 1024, 2048, 4096}) {
+        for (int L : {0, 64, 128, 256, 512, 1024, 2048, 4096}) {
             const cudaError_t e = cudaFuncSetAttribute((const void *)cols_kernel_steps(nsrc, L),
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
             if (e != cudaSuccess) return e;

@@ -675,7 +675,8 @@ __device__ __forceinline__ void fft_any(T (&v)[16], int L, int T_, int t, T *xb,
                                         D16 &&d16 = D16{})
 {
     if constexpr (sizeof(T) == 16) fft_f64<FWD, HALF>(v, L, T_, t, xb, twp);
-    else if constexpr (LC > 0) fft_ct<FWD, LC, HALF>(v, t, xb, twp, d16);
+    else if constexpr (LC >= 256) fft_ct<FWD, LC, HALF>(v, t, xb, twp, d16);
+    else if constexpr (LC > 0) fft_reg<FWD>(v, LC, LC / 16, t, xb, twp);   // the same code with a constant length
     else fft_reg<FWD>(v, L, T_, t, xb, twp);
 }
 

@@ -156,12 +156,16 @@ ColsKernel<R> cols_kernel_all(int nsrc, int L)
             if (L == 1024) return k_cols<R, 1, 1024, false>;
             if (L == 512) return k_cols<R, 1, 512, false>;
             if (L == 256) return k_cols<R, 1, 256, false>;
+            if (L == 128) return k_cols<R, 1, 128, false>;
+            if (L == 64) return k_cols<R, 1, 64, false>;
         } else {
             if (L == 4096) return k_cols<R, 2, 4096, false>;
             if (L == 2048) return k_cols<R, 2, 2048, false>;
             if (L == 1024) return k_cols<R, 2, 1024, false>;
             if (L == 512) return k_cols<R, 2, 512, false>;
             if (L == 256) return k_cols<R, 2, 256, false>;
+            if (L == 128) return k_cols<R, 2, 128, false>;
+            if (L == 64) return k_cols<R, 2, 64, false>;
         }
     }
     if (nsrc == 1) return k_cols<R, 1, 0, false>;
@@ -259,6 +263,8 @@ cudaError_t set_smem_limits(int max_optin)
                          (const void *)k_cols<float, 2, 0, false>,    (const void *)k_cols<float, 2, 4096, false>,
                          (const void *)k_cols<float, 2, 2048, false>, (const void *)k_cols<float, 2, 1024, false>,
                          (const void *)k_cols<float, 2, 512, false>,  (const void *)k_cols<float, 2, 256, false>,
+                         (const void *)k_cols<float, 1, 128, false>,  (const void *)k_cols<float, 1, 64, false>,
+                         (const void *)k_cols<float, 2, 128, false>,  (const void *)k_cols<float, 2, 64, false>,
                          (const void *)k_cols<double, 1, 0, false>,   (const void *)k_cols<double, 2, 0, false>,
                          (const void *)k_tabcols<float>,              (const void *)k_tabcols<double>};
     for (const void *fn : fns) {

@@ -424,6 +424,9 @@ cudaError_t launch_rows_fwd(const R *x0, const R *x1, int nsrc, void *xh, int nr
     if constexpr (sizeof(R) == 4) {
         if (nphi == 4096) go(k_rows_fwd<R, 2048>);
         else if (nphi == 2048) go(k_rows_fwd<R, 1024>);
+        else if (nphi == 256) go(k_rows_fwd<R, 128>);
+        else if (nphi == 128) go(k_rows_fwd<R, 64>);
+        else if (nphi == 64) go(k_rows_fwd<R, 32>);
         else go(k_rows_fwd<R, 0>);
     } else {
         go(k_rows_fwd<R, 0>);
@@ -669,6 +672,9 @@ cudaError_t launch_rows_inv(const void *oh, const RowOut &o, int nr, int nphi, c
     if constexpr (sizeof(R) == 4) {
         if (nphi == 4096) go(k_rows_inv<R, 2048>);
         else if (nphi == 2048) go(k_rows_inv<R, 1024>);
+        else if (nphi == 256) go(k_rows_inv<R, 128>);
+        else if (nphi == 128) go(k_rows_inv<R, 64>);
+        else if (nphi == 64) go(k_rows_inv<R, 32>);
         else go(k_rows_inv<R, 0>);
     } else {
         go(k_rows_inv<R, 0>);
@@ -680,6 +686,9 @@ cudaError_t set_row_smem_limits(int max_optin)
 {
     const void *fns[] = {(const void *)k_rows_fwd<float, 0>,      (const void *)k_rows_fwd<float, 2048>,
                          (const void *)k_rows_fwd<float, 1024>,   (const void *)k_rows_fwd<double, 0>,
+                         (const void *)k_rows_fwd<float, 128>,    (const void *)k_rows_fwd<float, 64>,
+                         (const void *)k_rows_fwd<float, 32>,     (const void *)k_rows_inv<float, 128>,
+                         (const void *)k_rows_inv<float, 64>,     (const void *)k_rows_inv<float, 32>,
                          (const void *)k_rows_inv<float, 0>,      (const void *)k_rows_inv<float, 2048>,
                          (const void *)k_rows_inv<float, 1024>,   (const void *)k_rows_inv<double, 0>,
                          (const void *)k_rows_fwd_tma<2048, 4>,   (const void *)k_rows_fwd_tma<1024, 4>,
