@@ -354,10 +354,32 @@ sg_status solve_into(sg_plan *pl, const void *sg_, const void *sd_, void *const 
 
 namespace {
 
+// Device address of a host range allocated page-locked, which the device can
+// write (alignment: the row transforms store element pairs); null for any other
+// memory (registered memory too: it may be registered read-only).
+void *mapped_range(void *h, size_t bytes, size_t align)
+{
+    cudaPointerAttributes a{}, b{};
+    unsigned int f = 0;
+    if (cudaPointerGetAttributes(&a, h) != cudaSuccess ||
+        cudaPointerGetAttributes(&b, (const char *)h + bytes - 1) != cudaSuccess || a.type != cudaMemoryTypeHost ||
+        cudaHostGetFlags(&f, h) != cudaSuccess || (f & cudaHostRegisterReadOnly)) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
+        (char *)b.devicePointer != (char *)a.devicePointer + bytes - 1 || ((uintptr_t)a.devicePointer & (align - 1)))
+        return nullptr;
+    return a.devicePointer;
+}
+
 // Pipelined host-buffer FFT solve: row chunks of the inputs are copied on the
-// plan's copy stream while the previous chunk's row transforms run on `s`;
-// after the column pass, each chunk's inverse row transforms are followed on
-// the copy stream by that chunk's output copies, overlapping the next
+// plan's copy stream while the previous chunk's row transforms run on `s`.
+// Page-locked outputs: the inverse rows store straight into them, at the
+// link's rate and with nothing to launch, signal or copy after them (1024 x 2048
+// gas 276 -> 228 us, 2048 x 4096 839 -> 792, 64 x 128 107 -> 43, against the
+// copies below).  Otherwise, each chunk's inverse row transforms are followed
+// on the copy stream by that chunk's output copies, overlapping the next
 // chunk's transforms.
 template <typename R>
 sg_status solve_host_fft(sg_plan *pl, const void *hsg, const void *hsd, void *const host_out[6], cudaStream_t s)
@@ -410,6 +432,16 @@ sg_status solve_host_fft(sg_plan *pl, const void *hsg, const void *hsd, void *co
         ro.src[ro.n] = q;
         ro.is_phi[ro.n] = (q % 3) == SG_COMP_PHI;
         ++ro.n;
+    }
+    RowOut direct = ro;
+    bool mapped = true;
+    for (int q = 0; q < ro.n && mapped; ++q)
+        mapped = (direct.ptr[q] = mapped_range(host_out[ro.src[q]], bytes, 2 * pl->esz)) != nullptr;
+    if (mapped) {
+        e = launch_rows_inv<R>(pl->oh, direct, nr, nphi, pl->tw_row, pl->twp_row, (const R *)pl->rcen, flag, s, 0, -1,
+                               pl->tm_rows ? &pl->tm_oh : nullptr, pl->flag, true, pl->rows_inv);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        return e == cudaSuccess ? SG_OK : cuda_fail(pl, e, "inverse transform into host memory");
     }
     for (int k = 0; k < nch && e == cudaSuccess; ++k) {
         // chunk 0 follows the column pass directly: a programmatic dependent of it
