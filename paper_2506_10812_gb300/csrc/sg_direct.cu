@@ -30,7 +30,7 @@
 // tile's largest scale heights; they lie around dj = 0) take the table
 // polynomials instead; every lane of a warp is on the same lag, so the two paths do not diverge.
 // Sums: 16 lags in a register, then Kahan-compensated.  Measured (solve): 128 x 256 gas + dust FP32
-// 112.6 -> 4.34 ms (0.99 Tpair/s; 15 operations at the FMA pipes' 37 Tlane/s would be 2.3), 61 x 150
+// 112.6 -> 3.5 ms (1.24 Tpair/s; 15 operations at the FMA pipes' 37 Tlane/s would be 2.3), 61 x 150
 // gas FP64 227 -> 6.89 ms (12.2 Gpair/s of the 21 that 27 operations allow), against one thread per
 // target with the Bessel functions by branch; errors against 64 bits as before (1.8e-7, 3.5e-15).
 //
@@ -378,17 +378,22 @@ k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__re
 }
 constexpr int kDirectRowMin = 8;
 
-// Targets per thread, warps per CTA and CTAs per cluster (source-row split).
-// A CTA's time is its pairs plus the lag tables it builds for them; the
-// device's is that times the CTAs an SM gets, stretched while the resident
-// warps times their independent targets are too few to cover the pipes'
-// latency.  KT: 1, 2, 4 (FP32), 1, 2 (FP64: registers).
+// Targets per thread, warps per CTA and CTAs per cluster (source-row split):
+// the shape with the least warp instructions on the fullest SM.  Per row pair
+// and lag tile a warp spends about 120 on barriers and limits, 35 per staged
+// source and 100 per lag of its threads' share, and per lag 3 and 16.5 a
+// target (FP32); CTAs of few warps wait at the barriers (half as long again with
+// one), and too few resident warps stretch it (24 fit, 16 with 4 targets each).
+// The choice is within 7 % of the best of 50 shapes on 27 x 27 to 256 x 512 discs:
+// 61 x 150 gas 0.145 ms with (1, 5, 8) against 0.22 with (1, 1, 8), 256 x 512 gas 13.1
+// with (4, 4, 8) against 16.7 with (1, 2, 8).  FP64: its instructions count alone,
+// 28 a pair and 60 a lag.  KT: 1, 2, 4 (FP32), 1, 2 (FP64: registers).
 struct DirectTile { int KT, W, S, nchunk; };
 static DirectTile direct_tile(int nr, int nphi, bool f64)
 {
     DirectTile best{1, 1, 1, 0};
     double best_t = 1e300;
-    const double lag = f64 ? 60.0 : 45.0, pair = f64 ? 28.0 : 18.0;
+    const double tiles = (nphi + DLT - 1) / DLT;
     for (int KT = 1; KT <= (f64 ? 2 : 4); KT *= 2)
         for (int W = 1; W <= DMAXT / 32; ++W) {
             const int TJ = 32 * W * KT;
@@ -396,9 +401,16 @@ static DirectTile direct_tile(int nr, int nphi, bool f64)
             const long long nchunk = (nphi + TJ - 1) / TJ;
             for (int S = 1; S <= 8 && S <= nr; S *= 2) {
                 const double ctas = std::ceil((double)nr * nchunk * S / 152.0);   // per SM
-                const double work = std::ceil((double)nr / S) * nphi * (TJ * pair + lag + 2.0 * KT * W * 32 / DLT * 30);
-                const double hide = std::min(ctas * W, 32.0) * std::min(KT, 2);
-                const double t = ctas * work * std::max(1.0, (f64 ? 12.0 : 24.0) / hide);
+                const double rows = std::ceil((double)nr / S);
+                double t;
+                if (f64) {
+                    const double work = rows * nphi * (TJ * 28.0 + 60.0 + 2.0 * KT * W * 32 / DLT * 30);
+                    t = ctas * work * std::max(1.0, 12.0 / (std::min(ctas * W, 32.0) * std::min(KT, 2)));
+                } else {
+                    const double share = (double)nphi / (32.0 * W);               // lags of a thread, over all tiles
+                    const double work = rows * W * (tiles * 120 + 35 * (KT * tiles + share) + 100 * share + nphi * (KT * 16.5 + 3));
+                    t = ctas * work * (1 + 0.5 / W) * std::max(1.0, 14.0 / std::min(ctas * W, KT == 4 ? 16.0 : 24.0));
+                }
                 if (t < best_t * 0.999) {
                     best_t = t;
                     best = {KT, W, S, (int)nchunk};
