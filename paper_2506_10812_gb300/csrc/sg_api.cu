@@ -220,7 +220,7 @@ sg_status build_tables(sg_plan *pl, cudaStream_t s)
             const double hb = b == 0 ? pl->p.h_g : pl->p.h_d;
             double *o64[3] = {eval, eval + lat, eval + 2 * lat};
             float *o32[3] = {nullptr, nullptr, nullptr};
-            e = launch_tab_eval(nr, nphi, pl->du, ha, hb, scale, kAlpha, !pl->f64, o64, o32, s);
+            e = launch_tab_eval(nr, nphi, pl->du, ha, hb, scale, kAlpha, o64, o32, s);
             for (int c = 0; c < 3 && e == cudaSuccess; ++c) {
                 e = launch_rows_fwd<double>(o64[c], nullptr, 1, spec, L, nphi, pl->tw_row64, pl->twp_row64,
                                             nullptr, false, s);
@@ -687,7 +687,7 @@ sg_status sg_kernel_table(sg_plan *pl, int pair, int comp, void *out_dev, void *
     float *o32[3] = {nullptr, nullptr, nullptr};
     if (pl->f64) o64[comp] = (double *)out_dev;
     else o32[comp] = (float *)out_dev;
-    cudaError_t e = launch_tab_eval(pl->p.nr, pl->p.nphi, pl->du, ha, hb, 1.0, 0.0, !pl->f64, o64, o32,
+    cudaError_t e = launch_tab_eval(pl->p.nr, pl->p.nphi, pl->du, ha, hb, 1.0, 0.0, o64, o32,
                                     (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(pl, e, "kernel table");
     return SG_OK;

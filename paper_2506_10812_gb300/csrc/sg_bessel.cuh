@@ -3,25 +3,13 @@
 // the two functions in Eq. "SG force kernel exact" (D) and Eq. "grav.
 // potential 2D" (K0e) of Rendon Restrepo et al. (2025), with X = d^2/8.
 //
-// CUDA's math library has no K0/K1, so they are evaluated here from three
-// published representations, each used where it converges fast:
-//   x < 2       ascending series (DLMF 10.31.1 and 10.31.2), FP64 only;
-//   x < x_asym  trapezoidal rule on the integral (DLMF 10.32.9 with
-//               w = 2 sqrt(x) sinh(t/2)):
-//                 K0e = x^-1/2     int_0^inf e^{-w^2/2} (1 + w^2/(4x))^-1/2 dw
-//                 D   = (2x^3/2)^-1 int_0^inf w^2 e^{-w^2/2} (1 + w^2/(4x))^-1/2 dw,
-//               both integrands positive (no cancellation for large x);
-//   x >= x_asym Hankel's asymptotic expansion (DLMF 10.40.2), the K1 - K0
-//               difference taken term by term (the leading terms cancel
-//               exactly, so no digits are lost).
-// Measured against 30-digit references: FP64 <= 1e-15, FP32 <= 2.3e-7
-// relative over their ranges.
-//
-// Where a function is evaluated per pair of cells the representations above
-// are too long: FP64 units run at 1/64 of the FP32 rate here, and a quadrature
-// is 24 reciprocal square roots.  bessel_table and the tail polynomials
-// (sg_bessel_tab.cuh) take one short polynomial per function instead: FP64
-// 12 or 10 multiply-adds, FP32 5 or 4.
+// CUDA's math library has no K0/K1, and FP64 units run at 1/64 of the FP32 rate
+// here, so each function is one short polynomial (sg_bessel_tab.cuh):
+//   x < 2^-20   ascending series (DLMF 10.31.1 and 10.31.2), FP64 only (rare);
+//   x < 16      quarter-octave tables, FP64 12 and FP32 5 multiply-adds;
+//   x >= 16     polynomials in 1/x (the tails), FP64 9 or 10, FP32 4.
+// (A quadrature of 24 reciprocal square roots and a Hankel series of 14
+// divisions took their place before: 128 x 256 plan and solve 15.5 ms, now 2.2.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -29,32 +17,6 @@
 #include "sg_bessel_tab.cuh"
 
 namespace sg {
-
-constexpr int NW64 = 24;        // FP64 nodes w_n = 0.4 n, n = 1..24 (e^{-w^2/2} < 1e-19 beyond)
-constexpr double HW64 = 0.4;
-constexpr int NW32 = 13;        // FP32 nodes w_n = 0.5 n, n = 1..13
-constexpr float HW32 = 0.5f;
-
-// Gaussian weights e^{-w_n^2/2} and w_n^2 e^{-w_n^2/2}, filled once per CTA.
-struct BesselWeights {
-    double g64[NW64 + 1], w2g64[NW64 + 1];
-    float g32[NW32 + 1], w2g32[NW32 + 1];
-};
-
-__device__ __forceinline__ void bessel_weights_init(BesselWeights &bw)
-{
-    for (int n = threadIdx.x; n <= NW64; n += blockDim.x) {
-        double w = HW64 * n;
-        bw.g64[n] = exp(-0.5 * w * w);
-        bw.w2g64[n] = w * w * bw.g64[n];
-    }
-    for (int n = threadIdx.x; n <= NW32; n += blockDim.x) {
-        double w = (double)HW32 * n;
-        double g = exp(-0.5 * w * w);
-        bw.g32[n] = (float)g;
-        bw.w2g32[n] = (float)(w * w * g);
-    }
-}
 
 // the ascending series, x < 2
 __device__ __forceinline__ void k0e_D_series(double x, double &k0e, double &D)
@@ -83,74 +45,6 @@ __device__ __forceinline__ void k0e_D_series(double x, double &k0e, double &D)
     const double ex = exp(x);
     k0e = ex * K0;
     D = ex * (K1 - K0);
-}
-
-__device__ __forceinline__ void k0e_D_f64(double x, const BesselWeights &bw, double &k0e, double &D)
-{
-    if (x < 2.0) {
-        k0e_D_series(x, k0e, D);
-    } else if (x < 40.0) {
-        const double q = 0.25 / x;
-        double s0 = 0.5, s1 = 0.0;
-#pragma unroll 4
-        for (int n = 1; n <= NW64; ++n) {
-            const double w = HW64 * n;
-            const double r = rsqrt(1.0 + w * w * q);
-            s0 += bw.g64[n] * r;
-            s1 += bw.w2g64[n] * r;
-        }
-        const double sx = sqrt(x);
-        k0e = HW64 * s0 / sx;
-        D = HW64 * s1 / (2.0 * x * sx);
-    } else {
-        const double s = sqrt(1.5707963267948966192 / x);
-        double t0 = 1.0, t1 = 1.0, s0 = 1.0, sd = 0.0;
-#pragma unroll
-        for (int k = 0; k < 14; ++k) {
-            const double o = (double)((2 * k + 1) * (2 * k + 1));
-            const double den = 1.0 / (8.0 * (k + 1) * x);
-            t0 *= -o * den;
-            t1 *= (4.0 - o) * den;
-            s0 += t0;
-            sd += t1 - t0;
-        }
-        k0e = s * s0;
-        D = s * sd;
-    }
-}
-
-// FP32 evaluation, valid for x >= 1.
-__device__ __forceinline__ void k0e_D_f32(float x, const BesselWeights &bw, float &k0e, float &D)
-{
-    if (x < 12.0f) {
-        const float q = 0.25f / x;
-        float s0 = 0.5f, s1 = 0.0f;
-#pragma unroll
-        for (int n = 1; n <= NW32; ++n) {
-            const float w = HW32 * n;
-            const float r = rsqrtf(fmaf(w * w, q, 1.0f));
-            s0 = fmaf(bw.g32[n], r, s0);
-            s1 = fmaf(bw.w2g32[n], r, s1);
-        }
-        const float rs = rsqrtf(x);
-        k0e = HW32 * s0 * rs;
-        D = HW32 * s1 * (0.5f * rs / x);
-    } else {
-        const float s = sqrtf(1.57079632679f / x);
-        const float ix = 1.0f / x;
-        float t0 = 1.0f, t1 = 1.0f, s0 = 1.0f, sd = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const float o = (float)((2 * k + 1) * (2 * k + 1));
-            const float den = ix * (1.0f / (8.0f * (k + 1)));
-            t0 *= -o * den;
-            t1 *= (4.0f - o) * den;
-            s0 += t0;
-            sd += t1 - t0;
-        }
-        k0e = s * s0;
-        D = s * sd;
-    }
 }
 
 // K0e(x) and E(x) = x D(x) from the quarter-octave tables, 2^-20 <= x < 16
@@ -205,8 +99,7 @@ __device__ __forceinline__ void bessel_tail(double z, double &S0, double &Q)
     }
 }
 
-// (K0e, D) at any x: table, tail or series (FP64; 10 to 14 multiply-adds a
-// function in place of the quadrature above).
+// (K0e, D) at any x: table, tail or series (FP64).
 __device__ __forceinline__ void k0e_D_short(double x, double &k0e, double &D)
 {
     if (x >= 16.0) {
@@ -221,6 +114,36 @@ __device__ __forceinline__ void k0e_D_short(double x, double &k0e, double &D)
         D = E / x;
     } else {
         k0e_D_series(x, k0e, D);                   // x < 2^-20, or not a number
+    }
+}
+
+// Pairs of one (target, source) row pair as a function of sg = sinh^2(Delta/2) +
+// sin^2(psi/2) = s^2 / (4 r r'), with eta = H^2 / (r r'), X = sg / (2 eta):
+//     P = A e^X K0(X) / (2 sqrt(pi) eta^1/2),   F = A D(X) / (8 sqrt(pi) eta^3/2).
+struct RowPair { double ix, teta, cP, cF, tP, tF; };
+__device__ __forceinline__ RowPair row_pair(double eta, double A)
+{
+    const double y = rsqrt(eta), c = A * 0.56418958354775628695 * y;       // 1 / sqrt(pi)
+    return {0.5 / eta, 2.0 * eta, 0.5 * c, 0.25 * c, 0.5 * A, 0.125 * A};
+}
+__device__ __forceinline__ void row_pair_eval(const RowPair &c, double sg, double &P, double &F)
+{
+    const double X = sg * c.ix, i1 = rsqrt(sg), isg = i1 * i1;
+    if (X >= 16.0) {
+        double S0, Q;
+        bessel_tail(c.teta * isg, S0, Q);
+        P = c.tP * i1 * S0;
+        F = c.tF * i1 * isg * Q;
+    } else if (bessel_in_table(X)) {
+        double k0e, E;
+        bessel_table(X, k0e, E);
+        P = c.cP * k0e;
+        F = c.cF * isg * E;
+    } else {                                       // X < 2^-20, or not a number
+        double k0e, D;
+        k0e_D_series(X, k0e, D);
+        P = c.cP * k0e;
+        F = c.cF * isg * (D * X);
     }
 }
 

@@ -35,11 +35,10 @@ cudaError_t set_row_smem_limits(int max_optin);   // the row transforms (sg_rows
 
 // Kernel-table evaluation (App. C lattice), one ordered pair (source aspect
 // ratio ha, target hb), all three components times scale * e^{alpha Delta},
-// written as [2 nr][nphi] arrays of type double (out64) or float (out32);
-// NULL skips.  mixed: evaluate the Bessel functions in FP32 where X >= 1
-// outside the nearest-neighbour stencil, FP64 elsewhere; otherwise FP64.
+// written as [2 nr][nphi] arrays of type double (out64) or float (out32),
+// evaluated in FP64; NULL skips.
 cudaError_t launch_tab_eval(int nr, int nphi, double du, double ha, double hb, double scale,
-                            double alpha, bool mixed, double *o64[3], float *o32[3], cudaStream_t s);
+                            double alpha, double *o64[3], float *o32[3], cudaStream_t s);
 
 // Row R2C of `nsrc` real [nrows][nphi] arrays x[a] (each row times
 // rscale[row] when rscale != NULL; row mean removed when dc) into packed

@@ -96,33 +96,12 @@ k_semi_table(int nr, int nphi, int lgG, const double2 *__restrict__ gi, const do
     double2 *xb = buf + (size_t)g * PL;
     const double2 li = gi[i - ip + nr - 1];
     {
-        const double inv_sqrt_pi = 0.56418958354775628695;
-        const double eta = sc[2 * g], A = sc[2 * g + 1], y = rsqrt(eta), ix = 0.5 / eta;
-        const double cP = A * (0.5 * inv_sqrt_pi) * y, cF = A * (0.25 * inv_sqrt_pi) * y;
+        const RowPair rp = row_pair(sc[2 * g], sc[2 * g + 1]);
 #pragma unroll 1
         for (int dj = t; dj <= N; dj += T) {
             const double2 lj = gj[dj];
-            const double sg = li.x + lj.x, X = sg * ix;                 // sigma = 4 sg
             double P = 0.0, F = 0.0;
-            if (!(i == ip && dj == 0)) {                                // self cell excluded
-                const double i1 = rsqrt(sg), isg = i1 * i1;
-                if (X >= 16.0) {
-                    double S0, Q;
-                    bessel_tail(2.0 * eta * isg, S0, Q);
-                    P = 0.5 * A * i1 * S0;
-                    F = 0.125 * A * i1 * isg * Q;
-                } else if (bessel_in_table(X)) {
-                    double k0e, E;
-                    bessel_table(X, k0e, E);
-                    P = cP * k0e;
-                    F = cF * isg * E;
-                } else {                                                // X < 2^-20, or not a number
-                    double k0e, D;
-                    k0e_D_series(X, k0e, D);
-                    P = cP * k0e;
-                    F = cF * isg * (D * X);
-                }
-            }
+            if (!(i == ip && dj == 0)) row_pair_eval(rp, li.x + lj.x, P, F);      // self cell excluded
             const double vR = F * (li.y + 2.0 * lj.x), vA = dj == N ? 0.0 : F * lj.y;
             double2 z, zm;                                              // at dj and at -dj
             if constexpr (PASS == 0) {
