@@ -108,12 +108,13 @@ typedef struct {
  * transform in phi, direct sum in r) takes scale heights that depend on r
  * only, H_a(r) = h_a r or any positive field whose rows are constant
  * (SG_ERR_ARG otherwise).  The pair kernel then depends on (r, r', phi - phi')
- * and the direct sum is, per azimuthal mode m, one complex nr x nr matrix
- * product.  The plan holds the phi-DFT of the exact pair kernel for every
- * (fluid pair, component, m, r, r'): semi_table size = nsrc^2 x 3 x nphi/2 x
- * nr^2 x (8 FP32 / 16 FP64), 25.8 GB for a 1024 x 2048 gas disc in FP32
- * (SG_ERR_OOM when it does not fit), built from FP64 kernel samples and row
- * transforms.  A solve is the FFT path's row transforms around one pass
+ * and the direct sum is, per azimuthal mode m, one nr x nr matrix product.
+ * The plan holds the phi-DFT of the exact pair kernel for every (fluid pair,
+ * component, m, r, r'); the kernel is even or odd in phi - phi', so each entry is
+ * one real number: nsrc^2 x 3 x (nphi/2 + 1) x nr^2 x (4 FP32 / 8 FP64) bytes,
+ * 12.9 GB for a 1024 x 2048 gas disc in FP32 (SG_ERR_OOM when it does not fit),
+ * built from FP64 kernel samples and row transforms.
+ * A solve is the FFT path's row transforms around one pass
  * that streams the tables; its result is the direct sum's (the same finite
  * sum, to the plan dtype's rounding).  sg_kernel_table is FFT only.        */
 sg_status sg_plan_create(sg_plan **out, const sg_params *p, void *stream);
