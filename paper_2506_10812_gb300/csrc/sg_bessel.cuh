@@ -9,7 +9,7 @@
 //   x < 16      quarter-octave tables, FP64 12 and FP32 5 multiply-adds;
 //   x >= 16     polynomials in 1/x (the tails), FP64 9 or 10, FP32 4.
 // (A quadrature of 24 reciprocal square roots and a Hankel series of 14
-// divisions took their place before: 128 x 256 plan and solve 15.5 ms, now 2.2.)
+// divisions took their place before: 128 x 256 semi-spectral plan and solve 15.6 ms, now 2.1.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -126,9 +126,10 @@ __device__ __forceinline__ RowPair row_pair(double eta, double A)
     const double y = rsqrt(eta), c = A * 0.56418958354775628695 * y;       // 1 / sqrt(pi)
     return {0.5 / eta, 2.0 * eta, 0.5 * c, 0.25 * c, 0.5 * A, 0.125 * A};
 }
-__device__ __forceinline__ void row_pair_eval(const RowPair &c, double sg, double &P, double &F)
+// i1 = 1 / sqrt(sg)
+__device__ __forceinline__ void row_pair_eval(const RowPair &c, double sg, double i1, double &P, double &F)
 {
-    const double X = sg * c.ix, i1 = rsqrt(sg), isg = i1 * i1;
+    const double X = sg * c.ix, isg = i1 * i1;
     if (X >= 16.0) {
         double S0, Q;
         bessel_tail(c.teta * isg, S0, Q);

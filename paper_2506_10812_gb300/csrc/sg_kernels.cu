@@ -113,7 +113,8 @@ k_tab_eval(int nr, int nphi, double du, double ha, double hb, double scale, doub
         double vP = 0.0, vR = 0.0, vA = 0.0;
         if (k != nr && !(k == 0 && j == 0)) {
             double F;
-            row_pair_eval(rp[x], sh2[x] + sp2, vP, F);
+            const double sg = sh2[x] + sp2;
+            row_pair_eval(rp[x], sg, rsqrt(sg), vP, F);
             vR = F * (em1[x] + 2.0 * sp2);
             vA = F * spsi;
         }

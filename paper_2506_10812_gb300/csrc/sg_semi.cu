@@ -60,6 +60,19 @@ __global__ void k_semi_geometry(int nr, int nphi, double du, double2 *gi, double
     }
 }
 
+// 1 / sqrt(sinh^2(Delta/2) + sin^2(psi/2)) for every lag, [|i - i'|][dj], dj <= nphi/2:
+// a function of the lags alone, read by every row pair and pair of fluids
+// in place of a reciprocal square root of about 10 FP64 instructions (128 x 256 gas +
+// dust plan and solve 2.23 -> 2.12 ms).
+__global__ void k_semi_lags(int nr, int N, const double2 *__restrict__ gi, const double2 *__restrict__ gj, double *i1)
+{
+    const int n = nr * (N + 1);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const int d = q / (N + 1), j = q - d * (N + 1);
+        i1[q] = rsqrt(gi[nr - 1 + d].x + gj[j].x);           // infinite at the self cell, which nothing reads
+    }
+}
+
 // Tables of one (source, target) pair of fluids: a CTA owns G source rows i'
 // of one target row i (blockIdx.y), n_phi / 16 threads each.  It samples the
 // three components for dj = 0 .. n_phi/2, mirrors them, transforms the row in
@@ -73,13 +86,13 @@ __global__ void k_semi_geometry(int nr, int nphi, double du, double2 *gi, double
 // parts are separable because W_Phi and W_r are even and W_phi odd.  An FP64
 // plan transforms W_Phi by itself (PASS 1) and W_r + W_phi (PASS 2), so that no
 // component takes on the rounding of a larger one.  128 x 256 gas + dust:
-// 15.5 -> 2.3 ms for a plan, a solve and the release (12.5 ms of it was sampling by
+// 15.6 -> 2.1 ms for a plan, a solve and the release (12.5 ms of it was sampling by
 // branch, 2.0 ms twelve real transforms).
 template <typename R, int PASS>
 __global__ void __launch_bounds__(512)
 k_semi_table(int nr, int nphi, int lgG, const double2 *__restrict__ gi, const double2 *__restrict__ gj,
-             const double *__restrict__ rc, const double *__restrict__ Ha, const double *__restrict__ Hb, double scale,
-             R *__restrict__ tab, const double2 *__restrict__ tw)
+             const double *__restrict__ i1, const double *__restrict__ rc, const double *__restrict__ Ha,
+             const double *__restrict__ Hb, double scale, R *__restrict__ tab, const double2 *__restrict__ tw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int T = nphi >> 4, N = nphi >> 1, G = 1 << lgG, PL = padded_len(nphi);
@@ -95,13 +108,14 @@ k_semi_table(int nr, int nphi, int lgG, const double2 *__restrict__ gi, const do
     __syncthreads();
     double2 *xb = buf + (size_t)g * PL;
     const double2 li = gi[i - ip + nr - 1];
+    const double *lag = i1 + (size_t)abs(i - ip) * (N + 1);
     {
         const RowPair rp = row_pair(sc[2 * g], sc[2 * g + 1]);
 #pragma unroll 1
         for (int dj = t; dj <= N; dj += T) {
             const double2 lj = gj[dj];
             double P = 0.0, F = 0.0;
-            if (!(i == ip && dj == 0)) row_pair_eval(rp, li.x + lj.x, P, F);      // self cell excluded
+            if (!(i == ip && dj == 0)) row_pair_eval(rp, li.x + lj.x, lag[dj], P, F);      // self cell excluded
             const double vR = F * (li.y + 2.0 * lj.x), vA = dj == N ? 0.0 : F * lj.y;
             double2 z, zm;                                              // at dj and at -dj
             if constexpr (PASS == 0) {
@@ -255,19 +269,20 @@ template <typename R>
 cudaError_t build_semi_tables(int nr, int nphi, int nsrc, double du, double dphi, double G, const double *rc_h,
                               const double *H_h[2], void *tab, const double *twp_h, size_t twp_n, cudaStream_t s)
 {
-    // scratch: the two lag tables, the transform's twiddles, the radii and the profiles
-    const size_t ngi = 2 * (size_t)(2 * nr), ngj = 2 * (size_t)nphi;
+    // scratch: the lag tables, the transform's twiddles, the radii and the profiles
+    const size_t ngi = 2 * (size_t)(2 * nr), ngj = 2 * (size_t)nphi, nlag = (size_t)nr * (nphi / 2 + 1);
     double *scr = nullptr;
-    cudaError_t e = cudaMalloc((void **)&scr, (ngi + ngj + twp_n + 3 * (size_t)nr) * sizeof(double));
+    cudaError_t e = cudaMalloc((void **)&scr, (ngi + ngj + twp_n + 3 * (size_t)nr + nlag) * sizeof(double));
     if (e != cudaSuccess) return e;
     double2 *gi = (double2 *)scr, *gj = (double2 *)(scr + ngi);
-    double *tw = scr + ngi + ngj, *rc = tw + twp_n, *H = rc + nr;
+    double *tw = scr + ngi + ngj, *rc = tw + twp_n, *H = rc + nr, *i1 = H + 2 * nr;
     e = cudaMemcpyAsync(tw, twp_h, twp_n * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(rc, rc_h, nr * sizeof(double), cudaMemcpyHostToDevice, s);
     for (int a = 0; a < nsrc && e == cudaSuccess; ++a)
         e = cudaMemcpyAsync(H + (size_t)a * nr, H_h[a], nr * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
         k_semi_geometry<<<(std::max(2 * nr, nphi) + 255) / 256, 256, 0, s>>>(nr, nphi, du, gi, gj);
+        k_semi_lags<<<(int)std::min<size_t>((nlag + 255) / 256, 152 * 16), 256, 0, s>>>(nr, nphi / 2, gi, gj, i1);
         e = cudaGetLastError();
     }
     // rows per CTA: 256 threads (512 for the longest rows) and at most the radial cells
@@ -281,7 +296,7 @@ cudaError_t build_semi_tables(int nr, int nphi, int nsrc, double du, double dphi
         for (int b = 0; b < nsrc && e == cudaSuccess; ++b) {
             R *dst = (R *)tab + (size_t)(a * nsrc + b) * 3 * (nphi / 2 + 1) * nr * nr;
             auto go = [&](auto kern) {
-                kern<<<grid, block, smem, s>>>(nr, nphi, lgG, gi, gj, rc, H + (size_t)a * nr, H + (size_t)b * nr, scale, dst,
+                kern<<<grid, block, smem, s>>>(nr, nphi, lgG, gi, gj, i1, rc, H + (size_t)a * nr, H + (size_t)b * nr, scale, dst,
                                                (const double2 *)tw);
             };
             if constexpr (sizeof(R) == 4) {
