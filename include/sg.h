@@ -89,7 +89,10 @@ typedef struct {
                                 h_d <= 0 means a gas-only disc                      */
     const void *H_g_field;   /* DIRECT and SEMISPECTRAL, optional: device [nr][nphi]
                                 H_g^sg(r,phi) in the plan dtype (copied at create);
-                                NULL = h_g r.  SEMISPECTRAL: every row constant    */
+                                NULL = h_g r.  SEMISPECTRAL: every row constant.
+                                DIRECT: the kernel takes H^2; a pair of two cells
+                                of zero height has none, and the target's outputs
+                                are NaN                                            */
     const void *H_d_field;   /* optional, as above for dust                         */
     double G;                /* gravitational constant (the paper's tests use 1)   */
     int32_t dtype;           /* SG_F32 or SG_F64                                    */

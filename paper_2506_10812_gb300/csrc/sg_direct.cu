@@ -174,9 +174,15 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
                 const R h = Hb[k] * q;
                 eb[k] = h * h;
             }
+            bool flat = false;
+#pragma unroll
+            for (int k = 0; k < KT; ++k) flat |= eb[k] == (R)0;
             for (int d0 = 0; d0 < nphi; d0 += DLT, ++tile) {
                 const int nlag = min(DLT, nphi - d0);
-                __syncthreads();                                 // the previous tile is done with
+                // the previous tile is done with.  A pair of two zero heights has no
+                // kernel (NaN, as in the short rows' kernel), which the tails at z = 0, the
+                // Newtonian limit, would hide: such a tile takes the pair by pair path.
+                const bool flats = __syncthreads_or(flat);
                 if (t == 0) s_amax[(tile + 1) & 1] = 0u;
                 // target slot x and lag d of the tile meet the source at window slot x - d + DLT - 1
                 float mx = 0.f;
@@ -188,7 +194,7 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
                     const R h = (Ha_f ? Ha_f[src] : ha * rr) * q, e = h * h;
                     win[w] = {(G * sig[src] * rr * rr * dudphi) * q, e};
                     const float ef = (float)e;
-                    nan |= ef != ef;
+                    nan |= ef != ef || (flats && e == (R)0);
                     mx = fmaxf(mx, ef);
                 }
                 const unsigned m = __reduce_max_sync(0xffffffffu, nan ? 0x7fc00000u : __float_as_uint(mx));
