@@ -88,6 +88,11 @@ std::vector<R> pass_twiddles(int L)
         const int (*rows)[2] = Rad == 16 ? r16 : Rad == 8 ? r8 : Rad == 4 ? r4 : r2;
         for (int q = 0; q < Rad / 2; ++q)
             for (int k = 0; k < Ns; ++k) {
+                if (q == 0 && 2 * k == Ns) {           // the right angle: 1, rotated by the kernel
+                    v.push_back((R)1);
+                    v.push_back((R)0);
+                    continue;
+                }
                 // exp(-2 pi i (p k / (Ns Rad) + j / 16)) as cosine and tangent, the fraction exact
                 const double a = 2.0 * M_PI * ((double)(rows[q][0] * k) / ((double)Ns * Rad) + rows[q][1] / 16.0);
                 v.push_back((R)std::cos(a));

@@ -315,17 +315,19 @@ __device__ __forceinline__ void final_pass(T (&v)[16], int t, int T_, int Ns, co
 // it.  A root is held as (c, t), w = c (1 + i t) (cosine and tangent, after Linzer and
 // Feig's multiply-add transforms): (u, v) = b (1 + i t) takes two multiply-adds, a + c (u, v) and
 // a - c (u, v) two each, six instructions and two roundings per value where a
-// complex product and two sums are eight and three.  (t may be as large as
-// 1.6e16, at a right angle: c t is the sine to rounding, and what the sum
-// b.x - t b.y then drops of b.x is c b.x < 1e-16 |b|.)  A
-// radix-16 pass is four such levels, the input twiddles w^r folded into them:
+// complex product and two sums are eight and three.  A right angle has no
+// tangent: only the first level of a pass meets it (w^(R/2) at k = Ns/2), where
+// b is rotated by register moves and the table holds the root 1 (bfly_first).
+// (The tangent of the rounded right angle, 1.6e16, overflowed for inputs above 1e291.)
+// All other tangents are below L / (2 pi), so that no input below 1e300 / L is
+// lost.  A radix-16 pass is four such levels, the input twiddles w^r folded into them:
 // level by level the roots are w^8; w^4 (and -i w^4); w^2 W8^k; w W16^k (k = 0,
 // 1, and so on; the upper half of each level is -i times the lower), so that a
 // pass reads 8 roots from its table, not 15, and is 192 instructions instead
 // of 228; the first pass, with constants, 148 instead of 168.
 // Table (pass_twiddles<double>): per pass of stride Ns, w = exp(-2 pi i k / (Ns R)),
 // rows of Ns roots: radix 16: w^8, w^4, w^2, w^2 W8, w, w W16, w W8, w W16^3;
-// radix 8: w^4, w^2, w, w W8; radix 4: w^2, w; radix 2: w.
+// radix 8: w^4, w^2, w, w W8; radix 4: w^2, w; radix 2: w; 1 where w^(R/2) is -i.
 // (a, b) <- (a + w b, a - w b), w conjugated for the inverse transform
 template <bool FWD> __device__ __forceinline__ void bfly(double2 &a, double2 &b, double2 w)
 {
@@ -333,6 +335,19 @@ template <bool FWD> __device__ __forceinline__ void bfly(double2 &a, double2 &b,
     const double u = fma(-t, b.y, b.x), v = fma(t, b.x, b.y);
     b = make_double2(fma(-w.x, u, a.x), fma(-w.x, v, a.y));
     a = make_double2(fma(w.x, u, a.x), fma(w.x, v, a.y));
+}
+// the first level of a pass: where `quarter`, the root is -i (the table's 1 times
+// it).  Integer selects, not FP64 instructions: the pipe that bounds the transform
+// is left alone.
+template <bool FWD> __device__ __forceinline__ void bfly_first(double2 &a, double2 &b, double2 w, bool quarter)
+{
+    const double2 x = b;
+    const int flip = quarter ? (int)0x80000000u : 0;
+    b.x = quarter ? x.y : x.x;
+    b.y = quarter ? x.x : x.y;
+    double &n = FWD ? b.y : b.x;                      // -i (x, y) = (y, -x), i (x, y) = (-y, x)
+    n = __hiloint2double(__double2hiint(n) ^ flip, __double2loint(n));
+    bfly<FWD>(a, b, w);
 }
 // the same with the root -i w
 template <bool FWD> __device__ __forceinline__ void bfly_mi(double2 &a, double2 &b, double2 w)
@@ -393,12 +408,15 @@ template <bool FWD, bool HALF> __device__ __forceinline__ void dft16_f64(double2
     bfly_mi<FWD>(v[14], v[15], W163);
     unreverse16(v);
 }
-// a later radix-16 pass; tp: its table row 0 at this thread's k
-template <bool FWD> __device__ __forceinline__ void pass16_f64(double2 (&v)[16], const double2 *__restrict__ tp, int Ns)
+// a later radix-16 pass at this thread's k; tp0: its table
+template <bool FWD>
+__device__ __forceinline__ void pass16_f64(double2 (&v)[16], const double2 *__restrict__ tp0, int k, int Ns)
 {
+    const double2 *tp = tp0 + k;
+    const bool quarter = 2 * k == Ns;
     const double2 w8 = __ldg(tp), w4 = __ldg(tp + Ns), w2 = __ldg(tp + 2 * Ns), w2a = __ldg(tp + 3 * Ns);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) bfly<FWD>(v[r], v[r + 8], w8);
+    for (int r = 0; r < 8; ++r) bfly_first<FWD>(v[r], v[r + 8], w8, quarter);
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         bfly<FWD>(v[r], v[r + 4], w4);
@@ -429,14 +447,16 @@ __device__ __forceinline__ void final_f64(double2 (&v)[16], int t, int T_, int N
     constexpr int Q = 16 / RL;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-        const double2 *tp = tp0 + ((t + T_ * q) & (Ns - 1));
+        const int k = (t + T_ * q) & (Ns - 1);
+        const double2 *tp = tp0 + k;
+        const bool quarter = 2 * k == Ns;
         double2 *x = v + q;                           // element r at x[r Q]
         if constexpr (RL == 2) {
-            bfly<FWD>(x[0], x[Q], __ldg(tp));
+            bfly_first<FWD>(x[0], x[Q], __ldg(tp), quarter);
         } else if constexpr (RL == 4) {
             const double2 w2 = __ldg(tp), w = __ldg(tp + Ns);
-            bfly<FWD>(x[0], x[2 * Q], w2);
-            bfly<FWD>(x[Q], x[3 * Q], w2);
+            bfly_first<FWD>(x[0], x[2 * Q], w2, quarter);
+            bfly_first<FWD>(x[Q], x[3 * Q], w2, quarter);
             bfly<FWD>(x[0], x[Q], w);
             bfly_mi<FWD>(x[2 * Q], x[3 * Q], w);
             const double2 y = x[Q];                   // order 0, 2, 1, 3
@@ -445,7 +465,7 @@ __device__ __forceinline__ void final_f64(double2 (&v)[16], int t, int T_, int N
         } else {
             const double2 w4 = __ldg(tp), w2 = __ldg(tp + Ns), w = __ldg(tp + 2 * Ns), wa = __ldg(tp + 3 * Ns);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) bfly<FWD>(x[r * Q], x[(r + 4) * Q], w4);
+            for (int r = 0; r < 4; ++r) bfly_first<FWD>(x[r * Q], x[(r + 4) * Q], w4, quarter);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 bfly<FWD>(x[r * Q], x[(r + 2) * Q], w2);
@@ -475,7 +495,7 @@ __device__ __forceinline__ void fft_f64(double2 (&v)[16], int L, int T_, int t, 
     const double2 *tp = twp;
     exchange16(v, t, T_, 1, xb);
     while (Ns * 16 <= L) {
-        pass16_f64<FWD>(v, tp + (t & (Ns - 1)), Ns);
+        pass16_f64<FWD>(v, tp, t & (Ns - 1), Ns);
         tp += 8 * Ns;
         if (Ns * 16 == L) return;
         exchange16(v, t, T_, Ns, xb);
