@@ -29,14 +29,22 @@ __device__ __forceinline__ C spec_at(const C *col, int k, int H, bool upper)
 // which set the time of every small column pass: 256 x 512 gas + dust 50 us,
 // 1024 x 2048 accelerations 48 us (LC: compile-time length, as in k_cols).
 // The two table columns of each source go to L2 while the forward transform
-// runs; Z*(L - k) comes through the exchange buffer.
+// runs; Z*(L - k) comes through the exchange buffer.  Long columns of two sources
+// leave the first one's products in the table area `park` (at least L elements, free
+// here) during the other's transform, instead of spilled: 1024 x 2048 67.6 against 69.6 us,
+// 512 x 1024 23.4 against 23.8, but 256 x 512 15.4 against 12.0.
+// Its transforms load every root: column 0 carries the axisymmetric part, which
+// dominates g_r, and the other columns' passes, which form nine of 15 roots as
+// products, make its error larger (axisymmetric discs of 128 to 2048 rows, g_r, mean
+// relative L2: 1.93e-7 so, 1.83e-7 with every root loaded).
 template <typename R, int NS, int LC>
 __device__ __noinline__ void col0_output(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab,
                                          cplx<R> *__restrict__ oh, int nr, int N, int q,
-                                         const cplx<R> *__restrict__ tw, cplx<R> *xb)
+                                         const cplx<R> *__restrict__ tw, cplx<R> *xb, cplx<R> *park)
 {
     using C = cplx<R>;
     const int L = LC > 0 ? LC : 2 * nr, T = L >> 4, H = L >> 1, P = tab_pitch(H);
+    constexpr bool PARK = NS == 2 && LC >= 1024;
     const int t = threadIdx.x, b = q / 3, c = q - 3 * b;
     if (t < 2 * NS)
         prefetch_l2_bulk(tab + (((size_t)((t >> 1) * NS + b) * 3 + c) * (N + 1) + (size_t)(t & 1) * N) * P,
@@ -51,7 +59,7 @@ __device__ __noinline__ void col0_output(const cplx<R> *__restrict__ sh, const c
         for (int e = 0; e < 8; ++e) v[e] = ld_cg_hint(col + blk(0, t + T * e, nr), l2_evict_last());
 #pragma unroll
         for (int e = 8; e < 16; ++e) v[e] = mkc<C>(0, 0);
-        fft_any<true, LC, true>(v, L, T, t, xb, tw);
+        fft_any<true, LC, true, true>(v, L, T, t, xb, tw);
         __syncthreads();                           // the transform's last exchange reads are done
 #pragma unroll
         for (int e = 0; e < 16; ++e) xb[pidx(t + T * e)] = v[e];
@@ -69,12 +77,18 @@ __device__ __noinline__ void col0_output(const cplx<R> *__restrict__ sh, const c
                 SN = cmul_mi(SN);
             }
             const C p = cscale(cadd(cmul(cadd(Z, Zm), S0), cmul(csub(Z, Zm), SN)), (R)0.5);
-            acc[e] = a == 0 ? p : cadd(acc[e], p);
+            if constexpr (PARK) {
+                // (acc is set in both turns, so that it does not live through the transform)
+                acc[e] = a == 0 ? p : cadd(park[k], p);
+                if (a == 0) park[k] = p;
+            } else {
+                acc[e] = a == 0 ? p : cadd(acc[e], p);
+            }
         }
         __syncthreads();                           // before the next transform rewrites the buffer
     }
     griddep_launch();
-    fft_any<false, LC>(acc, L, T, t, xb, tw);
+    fft_any<false, LC, false, true>(acc, L, T, t, xb, tw);
     C *o = oh + (size_t)q * N * nr;
 #pragma unroll
     for (int e = 0; e < 8; ++e) o[blk(0, t + T * e, nr)] = acc[e];
@@ -253,7 +267,7 @@ k_cols(const cplx<R> *__restrict__ sh, const cplx<R> *__restrict__ tab, cplx<R> 
     static_assert(!ST || sizeof(R) == 4, "per-step staging is FP32 only");
     constexpr bool PAIR = ST;
     if (m < 1) {
-        col0_output<R, NS, LC>(sh, tab, oh, nr, N, __ffs((int)outmask) - 1, tw, xb);
+        col0_output<R, NS, LC>(sh, tab, oh, nr, N, __ffs((int)outmask) - 1, tw, xb, tb);
         return;
     }
     if constexpr (PAIR) {

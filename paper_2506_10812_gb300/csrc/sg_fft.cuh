@@ -578,11 +578,17 @@ __device__ __forceinline__ void exchange_ct(T (&v)[16], int t, T *xb)
 //   spares the L1 data path 9 loads;
 //   final radix-RL pass: for each of its Q = 16 / RL butterflies, r = 1..4
 //   when RL = 8 (r = 5..7 as products of w4 and w1..w3), else r = 1..RL-1.
-template <int L, int Ns, typename T>
-__device__ __forceinline__ void load_pass_tw(const T *__restrict__ tp, int t, T (&b)[12])
+// FULL: every root is loaded and none is a product, the roundings of fft_reg.
+constexpr int pass_tw_len(bool full) { return full ? 15 : 12; }
+template <int L, int Ns, bool FULL, typename T>
+__device__ __forceinline__ void load_pass_tw(const T *__restrict__ tp, int t, T (&b)[pass_tw_len(FULL)])
 {
     constexpr int TT = L / 16;
-    if constexpr (Ns * 16 <= L) {
+    if constexpr (Ns * 16 <= L && FULL) {
+        const T *p = tp + (t & (Ns - 1));
+#pragma unroll
+        for (int r = 0; r < 15; ++r) b[r] = __ldg(p + r * Ns);
+    } else if constexpr (Ns * 16 <= L) {
         const T *p = tp + (t & (Ns - 1));
         b[0] = __ldg(p);
         b[1] = __ldg(p + Ns);
@@ -591,7 +597,7 @@ __device__ __forceinline__ void load_pass_tw(const T *__restrict__ tp, int t, T 
         b[4] = __ldg(p + 7 * Ns);
         b[5] = __ldg(p + 11 * Ns);
     } else {
-        constexpr int RL = L / Ns, Q = 16 / RL, NL = RL == 8 ? 4 : RL - 1;
+        constexpr int RL = L / Ns, Q = 16 / RL, NL = RL == 8 && !FULL ? 4 : RL - 1;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const T *p = tp + ((t + TT * q) & (Ns - 1));
@@ -610,13 +616,16 @@ template <bool FWD> struct RegDft16 {
     template <typename T> __device__ __forceinline__ void half(T (&v)[16]) const { dft16_half<FWD>(v); }
 };
 
-template <bool FWD, int L, int Ns, typename T, typename D16 = RegDft16<FWD>>
-__device__ __forceinline__ void fft_ct_pass(T (&v)[16], int t, T *xb, const T *__restrict__ tp, const T (&b)[12],
-                                            D16 &&d16 = D16{})
+template <bool FWD, int L, int Ns, bool FULL, typename T, typename D16 = RegDft16<FWD>>
+__device__ __forceinline__ void fft_ct_pass(T (&v)[16], int t, T *xb, const T *__restrict__ tp,
+                                            const T (&b)[pass_tw_len(FULL)], D16 &&d16 = D16{})
 {
     constexpr int TT = L / 16;
     if constexpr (Ns * 16 <= L) {
-        {
+        if constexpr (FULL) {
+#pragma unroll
+            for (int r = 1; r < 16; ++r) v[r] = twmul<FWD>(v[r], b[r - 1]);
+        } else {
             T w[16];
             w[1] = b[0];
             w[2] = b[1];
@@ -638,16 +647,16 @@ __device__ __forceinline__ void fft_ct_pass(T (&v)[16], int t, T *xb, const T *_
         }
         d16(v);
         if constexpr (Ns * 16 < L) {
-            T nb[12];
-            load_pass_tw<L, Ns * 16>(tp + 15 * Ns, t, nb);
+            T nb[pass_tw_len(FULL)];
+            load_pass_tw<L, Ns * 16, FULL>(tp + 15 * Ns, t, nb);
             exchange_ct<Ns, TT>(v, t, xb);
-            fft_ct_pass<FWD, L, Ns * 16>(v, t, xb, tp + 15 * Ns, nb, d16);
+            fft_ct_pass<FWD, L, Ns * 16, FULL>(v, t, xb, tp + 15 * Ns, nb, d16);
         }
     } else {
         constexpr int RL = L / Ns, Q = 16 / RL;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            if constexpr (RL == 8) {
+            if constexpr (RL == 8 && !FULL) {
                 T w[8];
 #pragma unroll
                 for (int r = 1; r <= 4; ++r) w[r] = b[q * 4 + r - 1];
@@ -675,27 +684,27 @@ __device__ __forceinline__ void fft_ct_pass(T (&v)[16], int t, T *xb, const T *_
 }
 
 // HALF: the inputs v[8..15] (x[L/2 ..]) are zero and the first pass skips them.
-template <bool FWD, int L, bool HALF = false, typename T, typename D16 = RegDft16<FWD>>
+template <bool FWD, int L, bool HALF = false, bool FULL = false, typename T, typename D16 = RegDft16<FWD>>
 __device__ __forceinline__ void fft_ct(T (&v)[16], int t, T *xb, const T *__restrict__ twp, D16 &&d16 = D16{})
 {
     static_assert(L >= 256 && (L & (L - 1)) == 0, "compile-time FFT needs a power of two >= 256");
     if constexpr (HALF) d16.half(v);
     else d16(v);
-    T b[12];
-    load_pass_tw<L, 16>(twp, t, b);
+    T b[pass_tw_len(FULL)];
+    load_pass_tw<L, 16, FULL>(twp, t, b);
     exchange_ct<1, L / 16>(v, t, xb);
-    fft_ct_pass<FWD, L, 16>(v, t, xb, twp, b, d16);
+    fft_ct_pass<FWD, L, 16, FULL>(v, t, xb, twp, b, d16);
 }
 
 // Compile-time length when LC > 0 (FP32), runtime length L otherwise (the
 // butterfly policy d16 applies to the compile-time lengths, the zero-half
-// pruning HALF to those and to FP64).
-template <bool FWD, int LC, bool HALF = false, typename T, typename D16 = RegDft16<FWD>>
+// pruning HALF to those and to FP64; FULL: no derived roots, see load_pass_tw).
+template <bool FWD, int LC, bool HALF = false, bool FULL = false, typename T, typename D16 = RegDft16<FWD>>
 __device__ __forceinline__ void fft_any(T (&v)[16], int L, int T_, int t, T *xb, const T *__restrict__ twp,
                                         D16 &&d16 = D16{})
 {
     if constexpr (sizeof(T) == 16) fft_f64<FWD, HALF>(v, L, T_, t, xb, twp);
-    else if constexpr (LC >= 256) fft_ct<FWD, LC, HALF>(v, t, xb, twp, d16);
+    else if constexpr (LC >= 256) fft_ct<FWD, LC, HALF, FULL>(v, t, xb, twp, d16);
     else if constexpr (LC > 0) fft_reg<FWD>(v, LC, LC / 16, t, xb, twp);   // the same code with a constant length
     else fft_reg<FWD>(v, L, T_, t, xb, twp);
 }
