@@ -6,7 +6,7 @@
 // CUDA's math library has no K0/K1, and FP64 units run at 1/64 of the FP32 rate
 // here, so each function is one short polynomial (sg_bessel_tab.cuh):
 //   x < 2^-20   ascending series (DLMF 10.31.1 and 10.31.2), FP64 only (rare);
-//   x < 16      quarter-octave tables, FP64 12 and FP32 5 multiply-adds;
+//   x < 16      quarter-octave tables, FP64 12 and FP32 6 multiply-adds and the last sum;
 //   x >= 16     polynomials in 1/x (the tails), FP64 9 or 10, FP32 4.
 // (A quadrature of 24 reciprocal square roots and a Hankel series of 14
 // divisions took their place before: 128 x 256 semi-spectral plan and solve 15.6 ms, now 2.1.)
@@ -55,11 +55,18 @@ __device__ __forceinline__ bool bessel_in_table(double x) { return x >= 0x1p-20 
 __device__ __forceinline__ void bessel_table(float x, float &k0e, float &E)
 {
     const int b = __float_as_int(x);
-    const float4 *c = reinterpret_cast<const float4 *>(&BT_32[(b >> 21) - 4 * (127 + BT_LO)][0][0]);
+    const int entry = (b >> 21) - 4 * (127 + BT_LO);
+    const float4 *c = reinterpret_cast<const float4 *>(&BT_32[entry][0][0]);
     const float t = __int_as_float((b & 0x007FFFFF) | 0x3F800000) - __int_as_float((b & 0x00600000) | 0x3F900000);
     const float4 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2);
-    k0e = fmaf(fmaf(fmaf(fmaf(fmaf(c1.y, t, c1.x), t, c0.w), t, c0.z), t, c0.y), t, c0.x);
-    E = fmaf(fmaf(fmaf(fmaf(fmaf(c2.w, t, c2.z), t, c2.y), t, c2.x), t, c1.w), t, c1.z);
+    const float4 l = __ldg(reinterpret_cast<const float4 *>(&BT_32L[entry][0]));
+    // the value is c_0 + (the rest, an eighth of it at most): rounded once, as if
+    // evaluated in 64 bits, within 0.2 of the last place
+    const float v = 64.0f * t * t, T6 = fmaf(fmaf(fmaf(32.0f, v, -48.0f), v, 18.0f), v, -1.0f);
+    const float k = fmaf(fmaf(fmaf(fmaf(c1.y, t, c1.x), t, c0.w), t, c0.z), t, c0.y);
+    const float e = fmaf(fmaf(fmaf(fmaf(c2.w, t, c2.z), t, c2.y), t, c2.x), t, c1.w);
+    k0e = c0.x + fmaf(k, t, fmaf(l.y, T6, l.x));
+    E = c1.z + fmaf(e, t, fmaf(l.w, T6, l.z));
 }
 __device__ __forceinline__ void bessel_table(double x, double &k0e, double &E)
 {

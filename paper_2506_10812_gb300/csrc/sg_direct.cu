@@ -84,14 +84,25 @@ template <typename R> constexpr size_t direct_smem(int T, int KT)
     return tab > red ? tab : red;
 }
 
-// 1 / sqrt(x) to rounding (the FP32 instruction alone is off by 2 ulp, and the
-// force takes its cube)
+// 1 / sqrt(x) to rounding (the FP32 instruction alone is off by 2 ulp)
 __device__ __forceinline__ float rsqrt_r(float x)
 {
     const float y = rsqrtf(x), e = fmaf(-x * y, y, 1.0f);
     return fmaf(0.5f * y, e, y);
 }
 __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
+
+// x / (2 sqrt(pi)), the common factor of a pair's terms, without the constant's own
+// rounding, which all pairs would share.  With w = m / (2 sqrt(pi) H) a pair is
+//     Phi term = w K0e,   force term = w E 2 / s^2 (r - r'),
+// one power of 1/H (its cube, in D = E / X, carried three times its rounding).
+__device__ __forceinline__ float over_2_sqrt_pi(float x)
+{
+    constexpr double c = 0.5 * 0.56418958354775628695;
+    constexpr float hi = (float)c, lo = (float)(c - (double)hi);
+    return fmaf(x, hi, x * lo);
+}
+__device__ __forceinline__ double over_2_sqrt_pi(double x) { return x * (0.5 * 0.56418958354775628695); }
 
 // One pair by its own scale height: (K0e, E) at z = 1 / X, any z.
 template <typename R>
@@ -253,14 +264,12 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
                         agp[k].add(sa[k]);
                     }
                 }
-                const R c_force = (R)(0.125 * 0.56418958354775628695);   // 1 / (8 sqrt(pi))
-                const R c_pot = (R)(0.5 * 0.56418958354775628695);       // 1 / (2 sqrt(pi))
 #pragma unroll 1
                 for (int d = 0; d < nlag; ++d) {
                     if (d == lo && lo < hi) d = hi;
                     if (d >= nlag) break;
                     if (i2 == i && d0 + d == 0) continue;        // self cell excluded
-                    const R iz = lagF[d].iz;
+                    const R iz = lagF[d].iz, hz = (R)0.5 * iz;
                     const Duo<R> g = lagN[d];
 #pragma unroll
                     for (int k = 0; k < KT; ++k) {
@@ -268,11 +277,11 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
                         const R eta = s.y + eb[k], z = eta * iz;
                         R k0e, E;
                         pair_bessel(z, k0e, E);
-                        const R invH = rsqrt_r((R)0.5 * eta);
-                        const R f = s.x * (E * z) * c_force * invH * invH * invH;   // G m K / s
+                        const R w = over_2_sqrt_pi(s.x * rsqrt_r((R)0.5 * eta));
+                        const R f = w * hz * E;                    // G m K / s
                         agr[k].add(f * g.x);
                         agp[k].add(f * g.y);
-                        aph[k].add(s.x * k0e * c_pot * invH);
+                        aph[k].add(w * k0e);
                     }
                 }
             }
@@ -331,8 +340,6 @@ k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__re
     const R hb = tgt == 0 ? h_g : h_d;
     const R Hb = valid ? (Hb_f ? Hb_f[tid] : hb * r) : (R)1;
     const R Hb2 = Hb * Hb;
-    const R c_force = (R)(0.125 * 0.56418958354775628695);   // 1 / (8 sqrt(pi))
-    const R c_pot = (R)(0.5 * 0.56418958354775628695);       // 1 / (2 sqrt(pi))
     Acc<R> agr, agp, aph;
     const int nsrc_fluids = sig_d ? 2 : 1;
     for (int a = 0; a < nsrc_fluids; ++a) {
@@ -368,11 +375,11 @@ k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__re
                 const R z = (R)8 * H2 / s2;
                 R k0e, E;
                 pair_bessel(z, k0e, E);
-                const R invH = rsqrt_r(H2);
-                const R f = s_m[q] * (E * z) * c_force * invH * invH * invH;   // G m K / s
-                agr.add(f * rr * (gi.y + (R)2 * gj.x));
-                agp.add(f * rr * gj.y);
-                aph.add(s_m[q] * k0e * c_pot * invH);
+                const R w = over_2_sqrt_pi(s_m[q] * rsqrt_r(H2));
+                const R f = w * ((R)2 * rr / s2) * E;        // G m K r' / s
+                agr.add(f * (gi.y + (R)2 * gj.x));
+                agp.add(f * gj.y);
+                aph.add(w * k0e);
             }
         }
     }
