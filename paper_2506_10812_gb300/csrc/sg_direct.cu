@@ -75,6 +75,10 @@ constexpr int DMAXT = 256;        // threads per CTA, at most
 template <typename R> struct __align__(16) LagFar { R iz, w1, wr, wp; };   // 4 / sigma, and the weights
 template <typename R> struct __align__(2 * sizeof(R)) Duo { R x, y; };
 
+// x times a constant held in two parts (the second is 0 in FP64): its rounding would
+// be one relative error, up to 6e-8, that all pairs share
+template <typename R> __device__ __forceinline__ R times(R x, Duo<R> c) { return fma(x, c.x, x * c.y); }
+
 // shared memory of a CTA of T threads and KT targets each; the partial sums
 // overlay the tables at the end
 template <typename R> constexpr size_t direct_smem(int T, int KT)
@@ -132,7 +136,7 @@ __global__ void __launch_bounds__(DMAXT)
 k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R *__restrict__ sig_d,
          const R *__restrict__ Hg, const R *__restrict__ Hd, R h_g, R h_d, int tgt, R *phi, R *gr,
          R *gphi, const typename pair_of<R>::type *__restrict__ geo_i,
-         const typename pair_of<R>::type *__restrict__ geo_j, const R *__restrict__ rcen, R dudphi,
+         const typename pair_of<R>::type *__restrict__ geo_j, const R *__restrict__ rcen, Duo<R> cell,
          unsigned int *flag)
 {
     using P2 = typename pair_of<R>::type;
@@ -203,7 +207,7 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
                     if (jj < 0) jj += nphi;
                     const size_t src = (size_t)i2 * nphi + jj;
                     const R h = (Ha_f ? Ha_f[src] : ha * rr) * q, e = h * h;
-                    win[w] = {(G * sig[src] * rr * rr * dudphi) * q, e};
+                    win[w] = {times(G * sig[src] * rr * rr, cell) * q, e};
                     const float ef = (float)e;
                     nan |= ef != ef || (flats && e == (R)0);
                     mx = fmaxf(mx, ef);
@@ -324,7 +328,7 @@ __global__ void __launch_bounds__(DT)
 k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__restrict__ sig_d,
                const R *__restrict__ Hg, const R *__restrict__ Hd, R h_g, R h_d, int tgt, R *phi, R *gr,
                R *gphi, const typename pair_of<R>::type *__restrict__ geo_i,
-               const typename pair_of<R>::type *__restrict__ geo_j, const R *__restrict__ rcen, R dudphi,
+               const typename pair_of<R>::type *__restrict__ geo_j, const R *__restrict__ rcen, Duo<R> cell,
                unsigned int *flag)
 {
     using P2 = typename pair_of<R>::type;
@@ -354,7 +358,7 @@ k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__re
                 const R rr = rcen[ii];
                 const R Ha = Ha_f ? Ha_f[src] : ha * rr;
                 s_r[threadIdx.x] = rr;
-                s_m[threadIdx.x] = G * sig[src] * rr * rr * dudphi;
+                s_m[threadIdx.x] = times(G * sig[src] * rr * rr, cell);
                 s_H2[threadIdx.x] = Ha * Ha;
                 s_i[threadIdx.x] = ii;
                 s_j[threadIdx.x] = jj;
@@ -441,12 +445,13 @@ cudaError_t launch_direct(int nr, int nphi, double r_in, double du, double G, co
 {
     (void)r_in;
     using P2 = typename pair_of<R>::type;
-    const double dphi = 2.0 * M_PI / nphi;
+    const double dphi = 2.0 * M_PI / nphi, area = du * dphi;
+    const Duo<R> cell = {(R)area, (R)(area - (double)(R)area)};
     if (nphi < kDirectRowMin) {
         const int ncell = nr * nphi;
         k_direct_short<R><<<(ncell + DT - 1) / DT, DT, 0, s>>>(
             nr, nphi, (R)G, sig_g, sig_d, Hg, Hd, (R)h_g, (R)h_d, tgt, phi, gr, gphi, (const P2 *)geo_i,
-            (const P2 *)geo_j, rcen, (R)(du * dphi), flag);
+            (const P2 *)geo_j, rcen, cell, flag);
         return cudaGetLastError();
     }
     const DirectTile d = direct_tile(nr, nphi, sizeof(R) == 8);
@@ -463,7 +468,7 @@ cudaError_t launch_direct(int nr, int nphi, double r_in, double du, double G, co
     cfg.numAttrs = 1;
     auto go = [&](auto kern) {
         return cudaLaunchKernelEx(&cfg, kern, nr, nphi, d.nchunk, (R)G, sig_g, sig_d, Hg, Hd, (R)h_g, (R)h_d, tgt, phi,
-                                  gr, gphi, (const P2 *)geo_i, (const P2 *)geo_j, rcen, (R)(du * dphi), flag);
+                                  gr, gphi, (const P2 *)geo_i, (const P2 *)geo_j, rcen, cell, flag);
     };
     cudaError_t e;
     if (d.KT == 1) e = go(k_direct<R, 1>);

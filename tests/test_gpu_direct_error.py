@@ -42,3 +42,19 @@ def test_thick_discs():
         a, b = solve_both(nr, nphi, *disc(nr, nphi, 0.5))
         err.append(float((a["phi_g"] - b["phi_g"]).norm() / b["phi_g"].norm()))
     assert np.mean(err) <= 3.93e-8, err
+
+
+def test_no_common_factor():
+    """Relative offset of the potential as a whole, on grids whose cell area du dphi
+    rounds to FP32 with an error of 5e-8 or more, thin and thick discs.  What all pairs
+    share would show in full; independent roundings of 6e-8 average out to less than
+    1.5e-8 over 28 rows and more."""
+    worst = 0.0
+    for nr, nphi in [(39, 80), (49, 64), (55, 112), (28, 112), (65, 96)]:
+        area = math.log(50.0) / nr * 2 * math.pi / nphi
+        assert abs(float(np.float32(area)) / area - 1) >= 5e-8, (nr, nphi)
+        for h in (0.03, 0.5):
+            a, b = solve_both(nr, nphi, *disc(nr, nphi, h))
+            a, b = a["phi_g"], b["phi_g"]
+            worst = max(worst, abs(float((a * b).sum() / (b * b).sum()) - 1))
+    assert worst <= 1.5e-8
