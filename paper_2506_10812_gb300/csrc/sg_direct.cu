@@ -25,14 +25,16 @@
 // sigma^-1/2 and the two sigma^-3/2 weights) once for all its targets, stages
 // the window of sources the tile meets, and then runs over dj: the lag's
 // entry is one broadcast, a target's source is at a fixed distance (conflict-
-// free), and a pair with z <= 1/16 costs 15 operations (FP32; 27 in FP64)
+// free), and a pair with z <= 1/16 costs 24 operations (FP32; 36 in FP64)
 // instead of a Bessel evaluation by branch (about 360).  Lags that may hold a larger z (a bound from the
 // tile's largest scale heights; they lie around dj = 0) take the table
 // polynomials instead; every lane of a warp is on the same lag, so the two paths do not diverge.
-// Sums: 16 lags in a register, then Kahan-compensated.  Measured (solve): 128 x 256 gas + dust FP32
-// 112.6 -> 3.5 ms (1.24 Tpair/s; 15 operations at the FMA pipes' 37 Tlane/s would be 2.3), 61 x 150
-// gas FP64 227 -> 6.89 ms (12.2 Gpair/s of the 21 that 27 operations allow), against one thread per
-// target with the Bessel functions by branch; errors against 64 bits as before (1.8e-7, 3.5e-15).
+// Every term is added with Kahan's compensation, 12 of the 24 operations.  (Sums of 16 lags
+// without it took 15 operations, 3.75 and 6.89 ms below, but left 0.56 units in the last place
+// where a compensated sum leaves 0.30.)  Measured (solve): 128 x 256 gas + dust FP32
+// 112.6 -> 4.62 ms (0.93 Tpair/s; 24 operations at the FMA pipes' 37 Tlane/s would be 2.8 ms), 61 x 150
+// gas FP64 227 -> 8.74 ms (9.6 Gpair/s of the 16 that 36 operations allow), against one thread per
+// target with the Bessel functions by branch; errors against 64 bits 1.2e-7 (1.8e-7 then) and 3.6e-15 (3.5e-15).
 //
 // The source rows are split over the CTAs of a cluster, whose partial sums
 // are added through distributed shared memory in rank order (no workspace, the
@@ -66,10 +68,16 @@ template <typename R> struct Acc {
         c = (t - s) - y;
         s = t;
     }
+    __device__ __forceinline__ void add(R a, R b)   // the same for a b, its rounding included
+    {
+        R y = fma(a, b, -c);
+        R t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
 };
 
 constexpr int DLT = 128;          // lags per tile
-constexpr int DGROUP = 16;        // lags per uncompensated partial sum
 constexpr int DMAXT = 256;        // threads per CTA, at most
 
 template <typename R> struct __align__(16) LagFar { R iz, w1, wr, wp; };   // 4 / sigma, and the weights
@@ -84,7 +92,7 @@ template <typename R> __device__ __forceinline__ R times(R x, Duo<R> c) { return
 template <typename R> constexpr size_t direct_smem(int T, int KT)
 {
     const size_t tab = DLT * (sizeof(LagFar<R>) + sizeof(Duo<R>)) + (size_t)(T * KT + DLT) * sizeof(Duo<R>);
-    const size_t red = (size_t)3 * T * KT * sizeof(R);
+    const size_t red = (size_t)6 * T * KT * sizeof(R);
     return tab > red ? tab : red;
 }
 
@@ -244,28 +252,18 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
                     }
                 }
                 const Duo<R> *wt = win + t + DLT - 1;
-                for (int g0 = lo; g0 < hi; g0 += DGROUP) {
-                    R sp[KT] = {}, sr[KT] = {}, sa[KT] = {};
-                    const int g1 = min(g0 + DGROUP, hi);
 #pragma unroll 4
-                    for (int d = g0; d < g1; ++d) {
-                        const LagFar<R> L = lagF[d];
-#pragma unroll
-                        for (int k = 0; k < KT; ++k) {
-                            const Duo<R> s = wt[k * T - d];
-                            R S0, Q;
-                            bessel_tail((s.y + eb[k]) * L.iz, S0, Q);
-                            sp[k] = fma(s.x, S0 * L.w1, sp[k]);
-                            Q *= s.x;
-                            sr[k] = fma(Q, L.wr, sr[k]);
-                            sa[k] = fma(Q, L.wp, sa[k]);
-                        }
-                    }
+                for (int d = lo; d < hi; ++d) {
+                    const LagFar<R> L = lagF[d];
 #pragma unroll
                     for (int k = 0; k < KT; ++k) {
-                        aph[k].add(sp[k]);
-                        agr[k].add(sr[k]);
-                        agp[k].add(sa[k]);
+                        const Duo<R> s = wt[k * T - d];
+                        R S0, Q;
+                        bessel_tail((s.y + eb[k]) * L.iz, S0, Q);
+                        aph[k].add(s.x, S0 * L.w1);
+                        Q *= s.x;
+                        agr[k].add(Q, L.wr);
+                        agp[k].add(Q, L.wp);
                     }
                 }
 #pragma unroll 1
@@ -291,14 +289,14 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
             }
         }
     }
-    // partial sums of the cluster's ranks, in rank order
-    R *red = reinterpret_cast<R *>(smem_raw);
+    // partial sums of the cluster's ranks, in rank order, each with its compensation
+    Duo<R> *red = reinterpret_cast<Duo<R> *>(smem_raw);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < KT; ++k) {
-        red[t + k * T] = aph[k].s;
-        red[TJ + t + k * T] = agr[k].s;
-        red[2 * TJ + t + k * T] = agp[k].s;
+        red[t + k * T] = {aph[k].s, -aph[k].c};
+        red[TJ + t + k * T] = {agr[k].s, -agr[k].c};
+        red[2 * TJ + t + k * T] = {agp[k].s, -agp[k].c};
     }
     cluster.sync();
     const R inv_r = (R)1 / r;
@@ -307,7 +305,11 @@ k_direct(int nr, int nphi, int nchunk, R G, const R *__restrict__ sig_g, const R
         const int c = x / TJ, j = j0 + x - c * TJ;
         if (j >= nphi) continue;
         Acc<R> v;
-        for (int p = 0; p < S; ++p) v.add(*cluster.map_shared_rank(red + x, p));
+        for (int p = 0; p < S; ++p) {
+            const Duo<R> s = *cluster.map_shared_rank(red + x, p);
+            v.add(s.x);
+            v.add(s.y);
+        }
         const R o = c == 0 ? -v.s : -v.s * inv_r;
         R *out = c == 0 ? phi : c == 1 ? gr : gphi;
         if (out) out[(size_t)i * nphi + j] = o;
@@ -396,15 +398,15 @@ k_direct_short(int nr, int nphi, R G, const R *__restrict__ sig_g, const R *__re
 constexpr int kDirectRowMin = 8;
 
 // Targets per thread, warps per CTA and CTAs per cluster (source-row split):
-// the shape with the least warp instructions on the fullest SM.  Per row pair
-// and lag tile a warp spends about 120 on barriers and limits, 35 per staged
-// source and 100 per lag of its threads' share, and per lag 3 and 16.5 a
-// target (FP32); CTAs of few warps wait at the barriers (half as long again with
-// one), and too few resident warps stretch it (24 fit, 16 with 4 targets each).
-// The choice is within 7 % of the best of 50 shapes on 27 x 27 to 256 x 512 discs:
-// 61 x 150 gas 0.145 ms with (1, 5, 8) against 0.22 with (1, 1, 8), 256 x 512 gas 13.1
-// with (4, 4, 8) against 16.7 with (1, 2, 8).  FP64: its instructions count alone,
-// 28 a pair and 60 a lag.  KT: 1, 2, 4 (FP32), 1, 2 (FP64: registers).
+// the shape with the least warp instructions on the fullest SM (152 of them).  Per row
+// pair and lag tile a warp spends about 72 on barriers and limits, 45 per staged
+// source and 160 per lag of its threads' share, and per lag 2 and 25.5 a
+// target (FP32); CTAs of few warps wait at the barriers (an eighth longer with one), and
+// fewer than 25 resident warps leave the pipes idle.  Fitted to 50 shapes on 8 discs of 24 x 48 to
+// 256 x 512, where the choice is within 8 % of the best: 53 x 603 gas 1.34 ms with (2, 2, 8)
+// against 1.96 with (4, 5, 8), 128 x 256 gas + dust 4.59 with (2, 4, 8) against 4.24 with (2, 2, 8).
+// FP64: its instructions count alone, 36 a pair and 60 a lag (within 11 % on 4
+// discs).  KT: 1, 2, 4 (FP32), 1, 2 (FP64: registers).
 struct DirectTile { int KT, W, S, nchunk; };
 static DirectTile direct_tile(int nr, int nphi, bool f64)
 {
@@ -421,12 +423,12 @@ static DirectTile direct_tile(int nr, int nphi, bool f64)
                 const double rows = std::ceil((double)nr / S);
                 double t;
                 if (f64) {
-                    const double work = rows * nphi * (TJ * 28.0 + 60.0 + 2.0 * KT * W * 32 / DLT * 30);
+                    const double work = rows * nphi * (TJ * 36.0 + 60.0 + 2.0 * KT * W * 32 / DLT * 30);
                     t = ctas * work * std::max(1.0, 12.0 / (std::min(ctas * W, 32.0) * std::min(KT, 2)));
                 } else {
                     const double share = (double)nphi / (32.0 * W);               // lags of a thread, over all tiles
-                    const double work = rows * W * (tiles * 120 + 35 * (KT * tiles + share) + 100 * share + nphi * (KT * 16.5 + 3));
-                    t = ctas * work * (1 + 0.5 / W) * std::max(1.0, 14.0 / std::min(ctas * W, KT == 4 ? 16.0 : 24.0));
+                    const double work = rows * W * (tiles * 72 + 45 * (KT * tiles + share) + 160 * share + nphi * (KT * 25.5 + 2));
+                    t = ctas * work * (1 + 0.12 / W) * std::max(1.0, 25.0 / (ctas * W));
                 }
                 if (t < best_t * 0.999) {
                     best_t = t;
