@@ -226,8 +226,8 @@ sg_status sg_stage_times(void *const *events, float *ms);
  * exits), so grids are limited to nr <= 1024 and nphi <= 4096; larger grids
  * return SG_ERR_UNSUPPORTED with a message on stderr.  The call allocates
  * and frees nothing.  Its first call in a CUDA context looks up the array's
- * device address (cudaGetSymbolAddress) for that context, so make that first
- * call before any stream capture; after cudaDeviceReset the next call looks
+ * device address (cudaGetSymbolAddress) and loads the kernels of every grid size
+ * and dtype for that context, so make that first call before any stream capture; after cudaDeviceReset the next call looks
  * it up again in the new context.  Every call shares the array and rewrites
  * the part it reads before reading it; calls whose GPU work overlaps (two
  * streams, two host threads) race on it, so serialise them.

@@ -502,6 +502,23 @@ __global__ void k_direct_geometry(int nr, int nphi, double r_in, double du, R *g
     }
 }
 
+// Load every kernel that a call may launch (CUDA loads a kernel at its first use,
+// which may take device memory): the grid's size chooses among them.
+static cudaError_t load_direct_kernels()
+{
+    const void *kernels[] = {(const void *)k_direct<float, 1>,        (const void *)k_direct<float, 2>,
+                             (const void *)k_direct<float, 4>,        (const void *)k_direct<double, 1>,
+                             (const void *)k_direct<double, 2>,       (const void *)k_direct_short<float>,
+                             (const void *)k_direct_short<double>,    (const void *)k_direct_geometry<float>,
+                             (const void *)k_direct_geometry<double>};
+    for (const void *k : kernels) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace sg
 
 namespace {
@@ -545,7 +562,7 @@ unsigned long long current_ctx_id()
 
 // Device address of the array in the current context: the lookup runs on the
 // first call in each context (it also makes the device's primary context
-// current when none is), later calls reuse it.
+// current when none is, and loads the kernels), later calls reuse it.
 cudaError_t noalloc_scratch(void **out)
 {
     int dev = -1;
@@ -558,6 +575,7 @@ cudaError_t noalloc_scratch(void **out)
     if (id == 0 || id != slot.ctx_id || !slot.ptr) {
         void *ptr = nullptr;
         e = cudaGetSymbolAddress(&ptr, g_sg_noalloc_scratch);
+        if (e == cudaSuccess) e = sg::load_direct_kernels();
         if (e != cudaSuccess) return e;
         slot.ptr = ptr;
         slot.ctx_id = current_ctx_id();            // nonzero once the lookup made a context current
@@ -622,7 +640,7 @@ extern "C" sg_status sg_direct_noalloc(const sg_params *p, const void *sigma_g, 
     void *scratch = nullptr;
     cudaError_t e = noalloc_scratch(&scratch);
     if (e != cudaSuccess) {
-        fprintf(stderr, "sg_direct_noalloc: cudaGetSymbolAddress: %s\n", cudaGetErrorString(e));
+        fprintf(stderr, "sg_direct_noalloc: scratch or kernels: %s\n", cudaGetErrorString(e));
         return SG_ERR_CUDA;
     }
     void *outs[6] = {phi_g, gr_g, gphi_g, phi_d, gr_d, gphi_d};
