@@ -177,7 +177,8 @@ sg_status sg_indirect(sg_plan *plan, const void *sigma_g, const void *sigma_d, d
 
 /* sg_solve with HOST buffers: inputs and outputs are host memory (pinned
  * memory gives full copy bandwidth).  The call copies the inputs to
- * plan-owned device buffers, solves, copies the requested outputs back and
+ * plan-owned device buffers, solves, copies the requested outputs back (an
+ * FFT plan writes them itself where all of them are page-locked allocations) and
  * synchronises `stream` before returning.  The first call allocates the
  * plan's staging buffers.                                                  */
 sg_status sg_solve_host(sg_plan *plan, const void *sigma_g, const void *sigma_d,

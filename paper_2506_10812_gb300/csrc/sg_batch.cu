@@ -114,7 +114,8 @@ __device__ bool wait_at_least(const unsigned *p, unsigned target, bool sys, cons
 
 // ------------------------------------------------------------ row R2C task
 // Rows rb G .. rb G + G - 1 of source `a` (rows past nr recompute row nr - 1
-// and store nothing).  Same arithmetic as k_rows_fwd.
+// and store nothing).  Same formulae as k_rows_fwd (FP64 rounded differently: the
+// plan kernels fold factors into multiply-adds).
 template <typename R, int NC>
 __device__ void task_fwd(const BatchDisc<R> &D, int a, int rb, unsigned char *smem)
 {
@@ -434,7 +435,7 @@ __device__ void task_col0(const BatchDisc<R> &D, unsigned char *smem)
 }
 
 // ------------------------------------------------- row C2R + epilogue task
-// Rows rb G .. of output slot q.  Same arithmetic as k_rows_inv.
+// Rows rb G .. of output slot q.  Same formulae as k_rows_inv (FP64 rounded differently).
 template <typename R, int NC>
 __device__ void task_inv(const BatchDisc<R> &D, int q, int rb, const BatchArgs &A, unsigned char *smem)
 {

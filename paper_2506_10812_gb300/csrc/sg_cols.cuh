@@ -26,8 +26,8 @@ __device__ __forceinline__ C spec_at(const C *col, int k, int H, bool upper)
 // the grid): NS forward transforms, the products and one inverse transform, so
 // no CTA's chain is longer than another column's.  One CTA for all outputs is
 // a chain of up to 3 NS (NS + 1) transforms with its table loads between them,
-// which set the time of every small column pass: 256 x 512 gas + dust 50 us,
-// 1024 x 2048 accelerations 48 us (LC: compile-time length, as in k_cols).
+// which set the time of every small column pass: solves of 256 x 512 gas + dust 43.0 ->
+// 25.7 us, 1024 x 2048 accelerations 75.4 -> 57.9 (LC: compile-time length, as in k_cols).
 // The two table columns of each source go to L2 while the forward transform
 // runs; Z*(L - k) comes through the exchange buffer.  Long columns of two sources
 // leave the first one's products in the table area `park` (at least L elements, free
@@ -123,7 +123,8 @@ constexpr int cols_min_blocks(int ns, bool f64, int lc, bool st)
 // series instead of NS + the outputs, for the forward transforms repeated by every
 // output.  Worth it while the chip is idle otherwise: a column CTA is a chain of
 // latencies, so as long as all CTAs of the split launch are resident at once
-// (FP32: 128 registers, 512 threads per SM) it is the chain that counts.  FP64
+// (FP32: 128 registers, 512 threads per SM; the shared memory of every default staging
+// allows as many; a GB300 has 152 SMs) it is the chain that counts.  FP64
 // instructions take a sub-partition 64 cycles a warp, so there the line is
 // one warp per sub-partition.
 inline bool cols_split(int N, int T, int nq, bool f64)

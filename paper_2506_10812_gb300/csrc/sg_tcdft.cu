@@ -389,7 +389,7 @@ cudaError_t launch_tc_stage(int engine, const void *in, void *out, long long cou
 cudaError_t launch_cols_tc(int engine, const void *sh, const void *tab, void *oh, int nr, int nphi, uint32_t outmask,
                            const void *tw_col, unsigned int *flag, cudaStream_t s)
 {
-    // column 0 on the FP32 column pass (one block)
+    // column 0 on the FP32 column pass (one block per requested output)
     cudaError_t e = launch_cols<float>(sh, tab, oh, nr, nphi, 1, outmask, tw_col, flag, s, 1);
     if (e != cudaSuccess || nphi / 2 < 2) return e;
     const int L = 2 * nr;
