@@ -170,12 +170,17 @@ struct SemiOut {
 // The stream of the tables bounds it: one real number per entry is half the
 // bytes of a complex table: 512 x 1024 gas 1.61 GB in 246 us (0.97 of the
 // measured HBM bandwidth), 3.23 GB in 537 us before.
+// FP32: a lane's four entries of a vector go to two sums in turn, so that neighbouring
+// rows, whose terms are the largest, do not follow one another in one chain (g_phi of
+// 7 grids, mean relative L2: 1.83e-7 in one chain, 1.79e-7 so). The registers are held to 4
+// (one source) or 3 CTAs per SM: 512 x 1024 gas 250 -> 249 us a solve, 512 x 512 gas + dust 565 -> 497,
+// 128 x 256 gas + dust 27.4 -> 29.4.
 template <typename R> struct vec_of;
 template <> struct vec_of<float> { using type = float4; };
 template <> struct vec_of<double> { using type = double2; };
 
 template <typename R, int NS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && NS == 1 ? 4 : 3)
 k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__restrict__ oh, int nr,
           int N, const __grid_constant__ SemiOut q)
 {
@@ -195,6 +200,7 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__
     const int ib = blockIdx.y * 32 + w * 4;
     const size_t plane = (size_t)nr * nr;
     R ar[4] = {0, 0, 0, 0}, ai[4] = {0, 0, 0, 0};
+    R br[4] = {0, 0, 0, 0}, bi[4] = {0, 0, 0, 0};         // FP32: every other entry of a vector
     // nr is a power of two >= 8, so a warp's four rows are all in the grid
     const size_t r0 = (size_t)ib * nr, r1 = r0 + nr, r2 = r1 + nr, r3 = r2 + nr;
 #pragma unroll 1
@@ -217,8 +223,9 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__
                     const R *tk = reinterpret_cast<const R *>(&t[k]);
 #pragma unroll
                     for (int x = 0; x < W; ++x) {
-                        ar[k] = fma(tk[x], s[x].x, ar[k]);
-                        ai[k] = fma(tk[x], s[x].y, ai[k]);
+                        R &xr = W == 4 && x % 2 ? br[k] : ar[k], &xi = W == 4 && x % 2 ? bi[k] : ai[k];
+                        xr = fma(tk[x], s[x].x, xr);
+                        xi = fma(tk[x], s[x].y, xi);
                     }
                 }
             }
@@ -233,6 +240,13 @@ k_semi_mv(const cplx<R> *__restrict__ sh, const R *__restrict__ tab, cplx<R> *__
                     ai[k] = fma(TN[rk[k] + ip], s.y, ai[k]);
                 }
             }
+        }
+    }
+    if constexpr (W == 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            ar[k] += br[k];
+            ai[k] += bi[k];
         }
     }
     griddep_launch();                                     // the inverse rows, late (as in the column pass)
